@@ -1,0 +1,42 @@
+"""Kernels chosen by size, type or alignment, at the edges of their ranges,
+against a plain restatement that rounds the same way (bit for bit), or the
+general kernel they stand in for."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2106_07136_gb300 as bd
+from gpu_helpers import dev, host
+
+pytestmark = pytest.mark.gpu
+
+
+def _warm_map_f32(p, level):
+    """Row-major float32 sums of each block's finite values, as the header states the map."""
+    b, h, w = p.shape
+    s = 1 << level
+    lo = s // 2
+    out = np.zeros((b, -(-h // s), -(-w // s)), np.float32)
+    for i in range(b):
+        for y in range(out.shape[1]):
+            for x in range(out.shape[2]):
+                v = p[i, max(y * s - lo, 0):y * s + lo, max(x * s - lo, 0):x * s + lo]
+                v = v[np.isfinite(v)]
+                if v.size:
+                    out[i, y, x] = np.add.accumulate(v, dtype=np.float32)[-1] / \
+                        np.float32(v.size) / np.float32(s)
+    return out
+
+
+@pytest.mark.parametrize("level,shape", [(1, (5, 7)), (2, (33, 65)), (3, (16, 24)), (3, (61, 301)),
+                                         (4, (97, 515)), (5, (120, 160)), (5, (135, 257)),
+                                         (6, (200, 333)), (7, (90, 1100)), (9, (70, 90)),
+                                         (13, (20, 30)), (14, (20, 30))])
+def test_warm_map_is_the_row_major_float32_mean(level, shape):
+    rng = np.random.default_rng(level * 1000 + shape[1])
+    p = rng.uniform(0.0, 60.0, size=(3, *shape)).astype(np.float32)
+    p[rng.random(p.shape) < 0.1] = np.nan
+    p[0, :3, :3] = np.inf
+    p[1, : shape[0] // 2] = np.nan
+    p[2, 1::5, 2::3] = -0.0
+    np.testing.assert_array_equal(host(bd.warm_map(dev(p), level)), _warm_map_f32(p, level))

@@ -40,3 +40,30 @@ def test_warm_map_is_the_row_major_float32_mean(level, shape):
     p[1, : shape[0] // 2] = np.nan
     p[2, 1::5, 2::3] = -0.0
     np.testing.assert_array_equal(host(bd.warm_map(dev(p), level)), _warm_map_f32(p, level))
+
+
+@pytest.mark.parametrize("ps,overlap", [(8, 0.75), (8, 0.5), (6, 0.6), (32, 0.9), (5, 0.0)])
+@pytest.mark.parametrize("count,shape", [(1, (33, 61)), (2, (67, 33)), (40, (161, 321))])
+def test_dis_densify_geometry(orc, ps, overlap, count, shape):
+    """DIS fusion over patch grids of other strides, with weights other than 1, dropped patches
+    and D* beyond the image; 5e-4 px as for the other DIS stages, the same unestimated pixels."""
+    h, w = shape
+    kw = dict(patch_size=ps, overlap=overlap, iterations=4, coarsest_scale=0, finest_scale=0,
+              fusion=bd._lib.BDIS_FUSION_DIS)
+    gp, op = bd.default_params(**kw), orc.OracleParams.make(**kw)
+    _, nx = bd.grid(w, ps, overlap)
+    _, ny = bd.grid(h, ps, overlap)
+    rng = np.random.default_rng(ps + count)
+    d = rng.uniform(-6, 40, (count, ny, nx)).astype(np.float32)
+    d[..., ::4] = np.round(d[..., ::4])  # whole samples: the last column is inside
+    weight = np.where(rng.random(d.shape) < 0.5, 1.0, rng.uniform(0.1, 2.0, d.shape))
+    weight = np.where(rng.random(d.shape) < 0.3, 0.0, weight).astype(np.float32)
+    d[weight == 0] = np.nan
+    L = rng.uniform(0, 255, (count, h, w)).astype(np.float32)
+    R = np.clip(L + rng.normal(0, 2, L.shape), 0, 255).astype(np.float32)
+    out = host(bd.densify_level((h, w), gp, dev(d), dev(weight), None, True, dev(L),
+                                bd.pack_right(dev(R))))
+    for i in {0, count - 1}:
+        ref = orc.densify_level((h, w), op, np.nan_to_num(d[i]), weight[i], None, True, L[i], R[i])
+        assert np.array_equal(np.isnan(out[i]), np.isnan(ref))
+        np.testing.assert_allclose(out[i], ref, atol=5e-4)

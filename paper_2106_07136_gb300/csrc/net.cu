@@ -20,8 +20,8 @@
 // default, or on mma.sync.m16n8k16; training uses mma.sync. The data-gradient of a layer is the same kernel run on the
 // output gradient with transposed, tap-flipped weights and the previous
 // layer's ReLU mask fused into the store; the weight-gradient is a GEMM with
-// rows = output channels, columns = (tap, input channel), K = pixels,
-// reduced across blocks with float atomics.
+// rows = output channels, columns = (tap, input channel), K = pixels, whose
+// blocks write partial sums that a second kernel adds in block order.
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -49,13 +49,6 @@ constexpr int kMasterCount = master_w_offset(kLayers);
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t *>(&v);
-}
-
-__device__ __forceinline__ uint32_t pack_raw(__nv_bfloat16 lo, __nv_bfloat16 hi) {
-  __nv_bfloat162 v;
-  v.x = lo;
-  v.y = hi;
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
@@ -829,106 +822,258 @@ __global__ void __launch_bounds__(kBandThreads, 1) net_forward_kernel(const Band
 
 // ------------------------------------------------------- weight gradient
 
-// dW[co][tap][ci] += sum_p G[p][co] * X[p shifted by tap][ci]; db[co] += sum_p G[p][co].
-// A block takes a run of 64 pixels at a time (grid-stride) and keeps the
-// whole COUT x (9 CIN) gradient in registers over its runs, then adds it to
-// global memory once. Rows = co (A = G^T), columns = (tap, ci), K = pixels.
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(128) conv_wgrad_kernel(
-    const __nv_bfloat16 *__restrict__ X, const __nv_bfloat16 *__restrict__ G, int dil, int H,
-    int W, long long total, float *__restrict__ dW, float *__restrict__ db) {
-  constexpr int PIX = 64;
-  constexpr int NCOL = 9 * CIN;          // GEMM columns
-  constexpr int NT = NCOL / 8;           // n-tiles
-  constexpr int MT = COUT / 16;          // m-tiles (COUT multiple of 16)
-  constexpr int NT_W = (NT + 3) / 4;     // n-tiles per warp
-  static_assert(COUT % 16 == 0 && CIN % 16 == 0, "tile");
-  __shared__ __align__(16) __nv_bfloat16 gs[PIX][COUT];
-  __shared__ __align__(16) __nv_bfloat16 xs[9][PIX][CIN];
-  __shared__ float dbs[COUT];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int g = lane >> 2, q = lane & 3;
-  const long long plane = (long long)H * W;
-  for (int c = threadIdx.x; c < COUT; c += blockDim.x) dbs[c] = 0.f;
-  float acc[MT][NT_W][4];
-#pragma unroll
-  for (int m = 0; m < MT; ++m)
-#pragma unroll
-    for (int n = 0; n < NT_W; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
-  float dbl = 0.f;  // bias partial of channel threadIdx.x (when < COUT)
-  for (long long base = (long long)blockIdx.x * PIX; base < total;
-       base += (long long)gridDim.x * PIX) {
-    __syncthreads();
-    // stage G (PIX x COUT) and the nine shifted copies of X (PIX x CIN), zero padded
-    for (int i = threadIdx.x; i < PIX * COUT / 2; i += blockDim.x) {
-      const int pix = i / (COUT / 2), c2 = (i - pix * (COUT / 2)) * 2;
-      const long long p = base + pix;
-      uint32_t v = 0u;
-      if (p < total) v = *reinterpret_cast<const uint32_t *>(G + p * COUT + c2);
-      *reinterpret_cast<uint32_t *>(&gs[pix][c2]) = v;
+// dW[co][tap][ci] = sum_p G[p][co] X[p shifted by tap][ci]; db[co] = sum_p
+// G[p][co], for all six layers in one launch, on mma.sync (M = co, N = (tap,
+// ci), K = pixels: 32 rows at most, which tcgen05's M of 64 or 128 would leave
+// half empty, and both operands pixel-major).
+//
+// Pixels are numbered in frames of (H + dil) x (W + dil) positions per image,
+// zero past the image: the zeros right of a row and below an image are also
+// those left of the next row and above the next image, so a tap is a constant
+// shift. A block takes tiles of 128 positions of one layer. Per tile it stages
+// G once and X as three segments of 128 + 2 dil positions (one per kernel
+// row, whatever the image width), two tiles in flight. ldmatrix.trans turns
+// the pixel-major rows into both operands' fragments; rows are swizzled so that
+// eight consecutive ones fall in distinct banks. A warp owns 8 input channels
+// (the first layer, with 2, is split over the warps by pixels instead) and all
+// nine taps; a block writes its totals to a partial buffer of its own, which
+// reduce_grad_kernel adds in a fixed order: no atomics, the same gradient every
+// time. Six launches that staged nine shifted copies of X word by word took
+// 500 us per 64 images of 40x30, of a gradient call's 780; it is now 310.
+constexpr int kWgTile = 128;
+constexpr int kWgRows = kWgTile + 2 * 4;  // rows of a segment at the largest dilation
+constexpr int kWgStage = (3 * kWgRows + kWgTile) * 64;  // bytes of one staged tile (X, then G)
+constexpr int kWgSmem = 2 * kWgStage, kWgPerSm = 3;  // 3 x 67 KB per SM
+constexpr int kPart = 32 * 9 * 32 + 32;  // floats of one block's partial: dW, then db
+
+struct WgradLayer {
+  const __nv_bfloat16 *X, *G;
+  int dil, first, blocks;  // blocks first .. first + blocks - 1 take the layer
+};
+struct WgradArgs {
+  WgradLayer layer[kLayers];
+  int H, W, count;
+  float *part;
+};
+
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+
+// byte offset of 16-byte chunk c of a row of C chunks (1 or 4)
+template <int C>
+__device__ __forceinline__ uint32_t wg_chunk(int row, int c) {
+  static_assert(C == 1 || C == 4, "chunks per row");
+  return C == 1 ? row * 16 : row * 64 + ((c ^ ((row >> 1) & 3)) << 4);
+}
+
+// One layer's tiles t = rank, rank + ranks, ... XS, GS: channels stored per
+// pixel; XC, GC: 16-byte chunks (8 channels) of them used; CO: real output
+// channels; CI: real input channels.
+template <int XS, int XC, int GS, int GC>
+__device__ __forceinline__ void wgrad_layer(const WgradArgs &args, const WgradLayer &ly,
+                                            uint8_t *smem, float *part) {
+  constexpr int MT = (GC + 1) / 2;       // 16-channel m-tiles
+  constexpr bool SPLIT = XC < 4;         // warps share the pixels, not the channels
+  static_assert(XC == 1 || XC == 4, "one warp per 8 input channels, or one group");
+  constexpr int CIW = XC * 8;            // input channels of the partial
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int H = args.H, W = args.W, dil = ly.dil, Wp = W + dil, Hp = H + dil;
+  const long long frame = (long long)Hp * Wp, total = frame * args.count;
+  const long long tiles = (total + kWgTile - 1) / kWgTile;
+  const int seg = kWgTile + 2 * dil, rank = (int)blockIdx.x - ly.first;
+  const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
+  const uint32_t goff = 3 * kWgRows * 64;
+  auto pixel = [&](long long q) -> long long {
+    if (q < 0 || q >= total) return -1;
+    int b, rem;
+    if (total < (1ll << 31)) {
+      b = (int)((unsigned)q / (unsigned)frame);
+      rem = (int)((unsigned)q - (unsigned)b * (unsigned)frame);
+    } else {
+      b = (int)(q / frame);
+      rem = (int)(q - (long long)b * frame);
     }
-    for (int i = threadIdx.x; i < 9 * PIX * CIN / 2; i += blockDim.x) {
-      const int tap = i / (PIX * CIN / 2);
-      const int rem = i - tap * (PIX * CIN / 2);
-      const int pix = rem / (CIN / 2), c2 = (rem - pix * (CIN / 2)) * 2;
-      const long long p = base + pix;
-      uint32_t v = 0u;
-      if (p < total) {
-        const int b = (int)(p / plane);
-        const int r2 = (int)(p - (long long)b * plane);
-        const int y = r2 / W + (tap / 3 - 1) * dil, x = r2 % W + (tap % 3 - 1) * dil;
-        if (y >= 0 && y < H && x >= 0 && x < W)
-          v = *reinterpret_cast<const uint32_t *>(X + (((long long)b * H + y) * W + x) * CIN + c2);
+    const int y = rem / Wp, x = rem - y * Wp;
+    return y < H && x < W ? ((long long)b * H + y) * W + x : -1;
+  };
+  auto stage = [&](long long tile, int buf) {
+    const uint32_t base = s0 + buf * kWgStage;
+    for (int i = tid; i < 3 * seg + kWgTile; i += 128) {
+      const bool isx = i < 3 * seg;
+      const int ty = i / seg, row = isx ? i - ty * seg : i - 3 * seg;
+      const long long q = tile * kWgTile + (isx ? (long long)(ty - 1) * dil * Wp - dil : 0) + row;
+      const long long p = pixel(q);
+      const int ok = p >= 0 ? 16 : 0;
+      if (isx) {
+#pragma unroll
+        for (int c = 0; c < XC; ++c)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                           base + wg_chunk<XC>(i, c)),
+                       "l"(ly.X + (p >= 0 ? p * XS + c * 8 : 0)), "r"(ok));
+      } else {
+#pragma unroll
+        for (int c = 0; c < GC; ++c)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                           base + goff + wg_chunk<GC>(row, c)),
+                       "l"(ly.G + (p >= 0 ? p * GS + c * 8 : 0)), "r"(ok));
       }
-      *reinterpret_cast<uint32_t *>(&xs[tap][pix][c2]) = v;
     }
-    __syncthreads();
-    if (threadIdx.x < COUT) {
-      float s = 0.f;
-      for (int pix = 0; pix < PIX; ++pix) s += __bfloat162float(gs[pix][threadIdx.x]);
-      dbl += s;
-    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  // the lane's ldmatrix row offsets: X rows of tap t for pixels 0 .. 31 of the
+  // tile, G rows for pixels 0 .. 15 (both advance by whole multiples of 32 rows,
+  // which leaves the swizzle as it is)
+  uint32_t xo[9], go[MT];
 #pragma unroll
-    for (int k0 = 0; k0 < PIX; k0 += 16) {
+  for (int t = 0; t < 9; ++t)
+    xo[t] = wg_chunk<XC>((t / 3) * seg + dil + (t % 3 - 1) * dil + lane, SPLIT ? 0 : warp);
 #pragma unroll
-      for (int m = 0; m < MT; ++m) {
-        // A[co][pix]: rows co = m*16 + g (+8), cols pix = k0 + 2q (+1) (+8)
-        const int co = m * 16 + g;
-        uint32_t a[4];
-        a[0] = pack_raw(gs[k0 + 2 * q][co], gs[k0 + 2 * q + 1][co]);
-        a[1] = pack_raw(gs[k0 + 2 * q][co + 8], gs[k0 + 2 * q + 1][co + 8]);
-        a[2] = pack_raw(gs[k0 + 2 * q + 8][co], gs[k0 + 2 * q + 9][co]);
-        a[3] = pack_raw(gs[k0 + 2 * q + 8][co + 8], gs[k0 + 2 * q + 9][co + 8]);
+  for (int m = 0; m < MT; ++m) {
+    const int mat = lane >> 3, chunk = m * 2 + (mat & 1);
+    go[m] = goff + wg_chunk<GC>((mat >> 1) * 8 + (lane & 7), GC == 1 ? 0 : chunk);
+  }
+  float acc[MT][9][4], adb[MT][4];
 #pragma unroll
-        for (int n = 0; n < NT_W; ++n) {
-          const int nt = warp * NT_W + n;
-          if (nt >= NT) break;
-          // B[pix][col]: col = nt*8 + g -> (tap, ci); rows pix = k0 + 2q (+1) (+8)
-          const int col = nt * 8 + g, tap = col / CIN, ci = col - tap * CIN;
-          uint32_t b[2];
-          b[0] = pack_raw(xs[tap][k0 + 2 * q][ci], xs[tap][k0 + 2 * q + 1][ci]);
-          b[1] = pack_raw(xs[tap][k0 + 2 * q + 8][ci], xs[tap][k0 + 2 * q + 9][ci]);
-          mma_bf16(acc[m][n], a, b);
+  for (int m = 0; m < MT; ++m) {
+    adb[m][0] = adb[m][1] = adb[m][2] = adb[m][3] = 0.f;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) acc[m][t][0] = acc[m][t][1] = acc[m][t][2] = acc[m][t][3] = 0.f;
+  }
+  const uint32_t ones[2] = {0x3f803f80u, 0x3f803f80u};
+  if (rank < tiles) stage(rank, 0);
+  int buf = 0;
+  for (long long tile = rank; tile < tiles; tile += ly.blocks, buf ^= 1) {
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();  // tile staged; the other buffer is read no more
+    if (tile + ly.blocks < tiles) stage(tile + ly.blocks, buf ^ 1);
+    const uint32_t base = s0 + buf * kWgStage;
+#pragma unroll 1
+    for (int k32 = SPLIT ? warp : 0; k32 < kWgTile / 32; k32 += SPLIT ? 4 : 1) {
+      uint32_t ga[MT][2][4];
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+          ldsm4t(ga[m][ks], base + go[m] + (k32 * 32 + ks * 16) * (GC * 16));
+          if (GC == 1) ga[m][ks][1] = ga[m][ks][3] = 0u;  // channels 8 .. 15 do not exist
         }
+      // a kernel row's three taps at a time: 3 MT independent MMAs before the
+      // accumulators come round again
+#pragma unroll
+      for (int ty = 0; ty < 3; ++ty) {
+        uint32_t xb[3][4];
+#pragma unroll
+        for (int tx = 0; tx < 3; ++tx)
+          ldsm4t(xb[tx], base + xo[ty * 3 + tx] + k32 * 32 * (XC * 16));
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+          for (int tx = 0; tx < 3; ++tx) {
+            const uint32_t bb[2] = {xb[tx][2 * ks], xb[tx][2 * ks + 1]};
+#pragma unroll
+            for (int m = 0; m < MT; ++m) mma_bf16(acc[m][ty * 3 + tx], ga[m][ks], bb);
+          }
       }
+      if (SPLIT || warp == 0)
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+          for (int m = 0; m < MT; ++m) mma_bf16(adb[m], ga[m][ks], ones);
     }
   }
-  // C[co][col]: acc[m][n][0..1] -> row m*16+g, cols nt*8 + 2q + {0,1}; [2..3] -> row +8
+  // acc[m][t][0..1] -> channel 16 m + g, inputs 2q, 2q + 1; [2..3] -> channel + 8
+  const int g = lane >> 2, q = lane & 3;
+  float *dst = part;
+  if (SPLIT) {  // the warps' sums meet in shared memory, one warp after the other
+    dst = reinterpret_cast<float *>(smem);
+    __syncthreads();
+  }
+  for (int turn = 0; turn < (SPLIT ? 4 : 1); ++turn) {
+    if (!SPLIT || turn == warp)
 #pragma unroll
-  for (int m = 0; m < MT; ++m)
+      for (int m = 0; m < MT; ++m)
 #pragma unroll
-    for (int n = 0; n < NT_W; ++n) {
-      const int nt = warp * NT_W + n;
-      if (nt >= NT) break;
-      const int col = nt * 8 + q * 2;
-      const int co = m * 16 + g;
-      // dW layout [co][tap][ci] == [co][col]
-      atomicAdd(dW + (long long)co * NCOL + col, acc[m][n][0]);
-      atomicAdd(dW + (long long)co * NCOL + col + 1, acc[m][n][1]);
-      atomicAdd(dW + (long long)(co + 8) * NCOL + col, acc[m][n][2]);
-      atomicAdd(dW + (long long)(co + 8) * NCOL + col + 1, acc[m][n][3]);
-    }
-  if (threadIdx.x < COUT) atomicAdd(db + threadIdx.x, dbl);
+        for (int h = 0; h < 2; ++h) {
+          const int co = m * 16 + h * 8 + g;
+          if (co >= GC * 8) continue;
+#pragma unroll
+          for (int t = 0; t < 9; ++t) {
+            float2 *o = reinterpret_cast<float2 *>(dst + (co * 9 + t) * CIW +
+                                                   (SPLIT ? 0 : warp * 8) + 2 * q);
+            const float2 old = SPLIT && turn ? *o : make_float2(0.f, 0.f);
+            *o = make_float2(old.x + acc[m][t][2 * h], old.y + acc[m][t][2 * h + 1]);
+          }
+          if (q == 0 && (SPLIT || warp == 0)) {
+            float *o = dst + kPart - 32 + co;
+            *o = (SPLIT && turn ? *o : 0.f) + adb[m][2 * h];
+          }
+        }
+    if (SPLIT) __syncthreads();
+  }
+  if (SPLIT) {
+    for (int i = tid; i < GC * 8 * 9 * CIW; i += 128) part[i] = dst[i];
+    if (tid < GC * 8) part[kPart - 32 + tid] = dst[kPart - 32 + tid];
+  }
+}
+
+__global__ void __launch_bounds__(128, kWgPerSm) conv_wgrad_kernel(const WgradArgs args) {
+  extern __shared__ __align__(128) uint8_t wg_smem[];
+  bdis::pdl_enter();
+  int l = 0;
+  while (l + 1 < kLayers && (int)blockIdx.x >= args.layer[l + 1].first) ++l;
+  float *part = args.part + (long long)blockIdx.x * kPart;
+  if (l == 0)
+    wgrad_layer<16, 1, 32, 4>(args, args.layer[0], wg_smem, part);
+  else if (l == 5)
+    wgrad_layer<32, 4, 16, 1>(args, args.layer[5], wg_smem, part);
+  else
+    wgrad_layer<32, 4, 32, 4>(args, args.layer[l], wg_smem, part);
+}
+
+struct LayerBlocks {
+  int first[kLayers], blocks[kLayers];
+};
+
+// Layer and position of master element i: weight (co, tap, ci), or bias (tap = 9).
+struct MasterAt {
+  int l, co, tap, ci;
+};
+__device__ __forceinline__ MasterAt master_at(int i) {
+  constexpr int first = master_w_offset(1), mid = master_w_offset(2) - first;
+  const int l = i < first ? 0 : 1 + (i - first) / mid;
+  const int cin = l == 0 ? 2 : 32, cout = l == 5 ? 1 : 32;
+  const int r = l == 0 ? i : i - first - (l - 1) * mid;
+  if (r >= cout * 9 * cin) return {l, r - cout * 9 * cin, 9, 0};
+  const int co = r / (9 * cin), m = r - co * 9 * cin;
+  return {l, co, m / cin, m % cin};
+}
+
+// The blocks' partial sums in master order: a block takes 32 elements, warp s
+// the partials s, s + 8, ..., and the eight sums are added in order.
+__global__ void __launch_bounds__(256) reduce_grad_kernel(const float *__restrict__ part,
+                                                          const LayerBlocks lb,
+                                                          float *__restrict__ grad) {
+  __shared__ float slice[8][32];
+  bdis::pdl_enter();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+  float sum = 0.f;
+  if (i < kMasterCount) {
+    const MasterAt m = master_at(i);
+    const int ciw = m.l == 0 ? 8 : 32;
+    const float *p = part + (long long)lb.first[m.l] * kPart +
+                     (m.tap == 9 ? kPart - 32 + m.co : (m.co * 9 + m.tap) * ciw + m.ci);
+#pragma unroll 8
+    for (int b = warp; b < lb.blocks[m.l]; b += 8) sum += __ldg(p + (long long)b * kPart);
+  }
+  slice[warp][lane] = sum;
+  __syncthreads();
+  if (warp == 0 && i < kMasterCount) {
+    for (int s = 1; s < 8; ++s) sum += slice[s][lane];
+    grad[i] = sum;
+  }
 }
 
 // ------------------------------------------------------ loss, weights, adam
@@ -978,8 +1123,7 @@ __global__ void bias_pad_kernel(const float *__restrict__ master, float *bias, i
   if (c < coutP) bias[c] = c < cout ? master[off + c] : 0.f;
 }
 
-// Adam on the master weights; gradients are gathered from the padded
-// per-layer gradient buffers.
+// Adam on the master weights.
 __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float *__restrict__ v,
                             const float *__restrict__ grad, int n, float lr, float b1, float b2,
                             float eps, float c1, float c2) {
@@ -991,20 +1135,6 @@ __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float 
   m[i] = mi;
   v[i] = vi;
   w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
-// Padded per-layer gradients [coutP][9][cinP] + [coutP] -> master order.
-__global__ void gather_grad_kernel(const float *__restrict__ dWp, const float *__restrict__ dbp,
-                                   float *__restrict__ grad, int off, int cin, int cout,
-                                   int cinP) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nw = cout * 9 * cin;
-  if (i < nw) {
-    const int co = i / (9 * cin), rem = i - co * 9 * cin, t = rem / cin, ci = rem - t * cin;
-    grad[off + i] = dWp[(co * 9 + t) * cinP + ci];
-  } else if (i < nw + cout) {
-    grad[off + i] = dbp[i - nw];
-  }
 }
 
 // Level-3 net output (channel 0 of z6) -> plain map.
@@ -1021,15 +1151,18 @@ struct bdis_net {
   int device = 0;
   // master weights and Adam state (f32, real channels, master order)
   float *w = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;
-  // per-layer padded bf16 weights, transposed copies, padded biases, padded grads
+  // per-layer padded bf16 weights, transposed copies, padded biases
   __nv_bfloat16 *wf[kLayers] = {}, *wb[kLayers] = {};
-  float *bias[kLayers] = {}, *dW[kLayers] = {}, *db[kLayers] = {};
+  float *bias[kLayers] = {};
   float *loss = nullptr;
   long long step = 0;
   // activations for `cap` pixels
   long long cap = 0;
-  __nv_bfloat16 *x0 = nullptr, *a[5] = {}, *gbuf[2] = {}, *g6 = nullptr;
+  // (gact[l]: gradient of layer l's output; the last layer's is g6)
+  __nv_bfloat16 *x0 = nullptr, *a[5] = {}, *gact[5] = {}, *g6 = nullptr;
   float *z6 = nullptr;
+  float *part = nullptr;  // partial weight gradients, one per block of conv_wgrad_kernel
+  int part_blocks = 0;
   // device word set when a forward kernel's bounded wait ran out
   int *fault = nullptr;
   unsigned *sync = nullptr;  // grid barrier counter of the fused inference kernel
@@ -1043,14 +1176,16 @@ namespace {
 void net_free_acts(bdis_net *n) {
   cudaFree(n->x0);
   for (auto &p : n->a) cudaFree(p);
-  for (auto &p : n->gbuf) cudaFree(p);
+  for (auto &p : n->gact) cudaFree(p);
   cudaFree(n->g6);
   cudaFree(n->z6);
+  cudaFree(n->part);
   n->x0 = nullptr;
   for (auto &p : n->a) p = nullptr;
-  for (auto &p : n->gbuf) p = nullptr;
+  for (auto &p : n->gact) p = nullptr;
   n->g6 = nullptr;
   n->z6 = nullptr;
+  n->part = nullptr;
   n->cap = 0;
 }
 
@@ -1085,8 +1220,11 @@ bdis_status net_reserve_pp(bdis_net *n, int h, int w, int count, cudaStream_t st
   return BDIS_OK;
 }
 
-bdis_status net_reserve(bdis_net *n, long long pixels) {
-  if (pixels <= n->cap) return BDIS_OK;
+// Activations for `pixels` pixels; with `train`, also the gradients of every
+// layer's output and the weight gradient's partial sums.
+bdis_status net_reserve(bdis_net *n, long long pixels, bool train) {
+  if (pixels <= n->cap && (!train || n->part)) return BDIS_OK;
+  pixels = std::max(pixels, n->cap);
   net_free_acts(n);
   cudaError_t e = cudaSuccess;
   auto alloc = [&](void **p, size_t bytes) {
@@ -1094,7 +1232,11 @@ bdis_status net_reserve(bdis_net *n, long long pixels) {
   };
   alloc((void **)&n->x0, pixels * 16 * 2);
   for (auto &p : n->a) alloc((void **)&p, pixels * 32 * 2);
-  for (auto &p : n->gbuf) alloc((void **)&p, pixels * 32 * 2);
+  if (train) {
+    for (auto &p : n->gact) alloc((void **)&p, pixels * 32 * 2);
+    n->part_blocks = kWgPerSm * bdis::device_sms() + kLayers;
+    alloc((void **)&n->part, sizeof(float) * kPart * n->part_blocks);
+  }
   alloc((void **)&n->g6, pixels * 16 * 2);
   alloc((void **)&n->z6, pixels * 16 * 4);
   if (e != cudaSuccess) {
@@ -1300,41 +1442,49 @@ cudaError_t forward(bdis_net *n, const float *L3, const float *R3, int r_stride,
   return cudaGetLastError();
 }
 
-// Backward through all layers into the padded gradient buffers (zeroed here).
+// Backward through all layers: the data gradients, layer by layer, then every
+// layer's weight gradient in one launch and the sum of its partials.
 cudaError_t backward(bdis_net *n, int H, int W, long long total, cudaStream_t st) {
-  cudaError_t e = cudaSuccess;
-  for (int l = 0; l < kLayers && e == cudaSuccess; ++l) {
-    e = cudaMemsetAsync(n->dW[l], 0, sizeof(float) * kCoutP[l] * 9 * kCinP[l], st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(n->db[l], 0, sizeof(float) * kCoutP[l], st);
-  }
-  if (e != cudaSuccess) return e;
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, n->device);
-  const unsigned wblocks = (unsigned)std::min<long long>((total + 63) / 64, (long long)sms * 4);
-  // layer 6 (linear): gradient g6 of z6
-  conv_wgrad_kernel<32, 16><<<wblocks, 128, 0, st>>>(n->a[4], n->g6, kDil[5], H, W, total,
-                                                     n->dW[5], n->db[5]);
   // g5 = (W6^T g6) * relu'(a5)
   conv<16, 32, kBwdDataMasked>(n->g6, n->wb[5], nullptr, kDil[5], H, W, total, n->a[4],
-                               n->gbuf[0], n->fault, st);
-  int cur = 0;
-  for (int l = 4; l >= 1; --l) {
-    // gradient of layer l (0-based) output is gbuf[cur]; its input is a[l-1]
-    conv_wgrad_kernel<32, 32><<<wblocks, 128, 0, st>>>(n->a[l - 1], n->gbuf[cur], kDil[l], H, W,
-                                                       total, n->dW[l], n->db[l]);
-    conv<32, 32, kBwdDataMasked>(n->gbuf[cur], n->wb[l], nullptr, kDil[l], H, W, total,
-                                 n->a[l - 1], n->gbuf[cur ^ 1], n->fault, st);
-    cur ^= 1;
-  }
-  conv_wgrad_kernel<16, 32><<<wblocks, 128, 0, st>>>(n->x0, n->gbuf[cur], kDil[0], H, W, total,
-                                                     n->dW[0], n->db[0]);
+                               n->gact[4], n->fault, st);
+  for (int l = 4; l >= 1; --l)
+    conv<32, 32, kBwdDataMasked>(n->gact[l], n->wb[l], nullptr, kDil[l], H, W, total,
+                                 n->a[l - 1], n->gact[l - 1], n->fault, st);
+  // Blocks per layer: as many in all as run at once, in proportion to the layers' work (a
+  // tile of the first or last layer is a fraction of a middle one's)
+  static const double kCost[kLayers] = {0.4, 1, 1, 1, 1, 0.6};
+  WgradArgs wa{};
+  LayerBlocks lb{};
+  const int count = (int)(total / ((long long)H * W));
+  long long tiles[kLayers];
+  double work = 0;
   for (int l = 0; l < kLayers; ++l) {
-    const int cnt = kCout[l] * 9 * kCin[l] + kCout[l];
-    gather_grad_kernel<<<nblocks(cnt, 256), 256, 0, st>>>(n->dW[l], n->db[l], n->grad,
-                                                          master_w_offset(l), kCin[l], kCout[l],
-                                                          kCinP[l]);
+    tiles[l] = ((long long)(H + kDil[l]) * (W + kDil[l]) * count + kWgTile - 1) / kWgTile;
+    work += tiles[l] * kCost[l];
   }
-  return cudaGetLastError();
+  int blocks = 0;
+  for (int l = 0; l < kLayers; ++l) {
+    const double share = (n->part_blocks - kLayers) * tiles[l] * kCost[l] / work;
+    lb.first[l] = blocks;
+    lb.blocks[l] = (int)std::max(1ll, std::min(tiles[l], (long long)share));
+    blocks += lb.blocks[l];
+    wa.layer[l] = {l ? n->a[l - 1] : n->x0, l < 5 ? n->gact[l] : n->g6, kDil[l], lb.first[l],
+                   lb.blocks[l]};
+  }
+  wa.H = H;
+  wa.W = W;
+  wa.count = count;
+  wa.part = n->part;
+  cudaError_t e = cudaFuncSetAttribute(conv_wgrad_kernel,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
+  if (e == cudaSuccess)
+    e = bdis::launch_maybe_overlapped(conv_wgrad_kernel, dim3((unsigned)blocks), dim3(128),
+                                      (size_t)kWgSmem, st, wa);
+  if (e == cudaSuccess)
+    e = bdis::launch_maybe_overlapped(reduce_grad_kernel, dim3(nblocks(kMasterCount, 32)),
+                                      dim3(256), 0, st, (const float *)n->part, lb, n->grad);
+  return e;
 }
 
 void net_release(bdis_net *n) {
@@ -1352,8 +1502,6 @@ void net_release(bdis_net *n) {
     cudaFree(n->wf[l]);
     cudaFree(n->wb[l]);
     cudaFree(n->bias[l]);
-    cudaFree(n->dW[l]);
-    cudaFree(n->db[l]);
   }
   delete n;
 }
@@ -1375,7 +1523,7 @@ bdis_status net_forward_on(bdis_net *n, const float *L, const float *R, int r_st
       if (forward_pp(n, L, R, r_stride, h, w, count, out, st)) return record_cuda(cudaGetLastError());
     }
   }
-  bdis_status s = net_reserve(n, total);
+  bdis_status s = net_reserve(n, total, false);
   if (s != BDIS_OK) return s;
   cudaError_t e = forward(n, L, R, r_stride, h, w, total, st);
   if (e == cudaSuccess) {
@@ -1420,8 +1568,6 @@ bdis_status bdis_net_create(int device, const float *weights, bdis_net **out) {
     alloc((void **)&n->wf[l], 2 * kCoutP[l] * 9 * kCinP[l]);
     if (l > 0) alloc((void **)&n->wb[l], 2 * kCoutP[l] * 9 * kCinP[l]);
     alloc((void **)&n->bias[l], sizeof(float) * kCoutP[l]);
-    alloc((void **)&n->dW[l], sizeof(float) * kCoutP[l] * 9 * kCinP[l]);
-    alloc((void **)&n->db[l], sizeof(float) * kCoutP[l]);
   }
   if (e == cudaSuccess) e = cudaMemcpy(n->w, weights, wb, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(n->m, 0, wb);
@@ -1454,7 +1600,7 @@ bdis_status bdis_net_gradient(bdis_net *n, const float *L3, const float *R3, int
       (r_stride != 1 && r_stride != 2))
     return BDIS_E_INVALID_ARG;
   const long long total = (long long)width * height * count;
-  bdis_status s = net_reserve(n, total);
+  bdis_status s = net_reserve(n, total, true);
   if (s != BDIS_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = forward(n, L3, R3, r_stride, height, width, total, st);

@@ -7,6 +7,7 @@ import torch
 
 import paper_2106_07136_gb300 as bd
 from gpu_helpers import dev, host
+from oracle import net_oracle as no
 
 pytestmark = pytest.mark.gpu
 
@@ -67,3 +68,29 @@ def test_dis_densify_geometry(orc, ps, overlap, count, shape):
         ref = orc.densify_level((h, w), op, np.nan_to_num(d[i]), weight[i], None, True, L[i], R[i])
         assert np.array_equal(np.isnan(out[i]), np.isnan(ref))
         np.testing.assert_allclose(out[i], ref, atol=5e-4)
+
+
+@pytest.mark.parametrize("count,h,w", [(8, 1, 1), (2, 2, 129), (4, 33, 5), (2, 9, 300), (16, 31, 41)])
+def test_weight_gradient_of_a_batch_is_the_mean_of_its_images(count, h, w):
+    """Images smaller than a tile, narrower than a tap, wider than a tile, and tiles that hold
+    several images. For a power of two of images every activation and activation gradient of the
+    batch is that of the image alone (scaled exactly), so the gradients differ by the order of
+    32-bit sums only: 1e-5 of each layer's norm. The gradient is the same every time."""
+    rng = np.random.default_rng(w)
+    L = rng.uniform(0, 255, (count, h, w)).astype(np.float32)
+    R = rng.uniform(0, 255, (count, h, w)).astype(np.float32)
+    label = rng.uniform(0, 4, (count, h, w)).astype(np.float32)
+    label[rng.random(label.shape) < 0.1] = np.nan
+    net = bd.ProposalNet(bd.net_init_weights(seed=w))
+    loss, g = net.gradient(dev(L), dev(R), dev(label))
+    assert np.array_equal(net.gradient(dev(L), dev(R), dev(label))[1], g)
+    each = [net.gradient(dev(L[i]), dev(R[i]), dev(label[i])) for i in range(count)]
+    net.close()
+    assert abs(loss - np.mean([e[0] for e in each])) <= 1e-5 * loss
+    mean = np.mean([e[1].astype(np.float64) for e in each], axis=0)
+    off = 0
+    for ci, co in no.CHANNELS:
+        n = co * 9 * ci + co
+        a, b = g[off:off + n], mean[off:off + n]
+        assert np.linalg.norm(a - b) <= 1e-5 * np.linalg.norm(b), (ci, co)
+        off += n

@@ -512,9 +512,11 @@ int bdis_net_weight_count(void);
  * 3x3 tap's operand a shifted window of it, accumulators in tensor memory,
  * the next band's copy overlapping the epilogue; 2 = the per-tile tcgen05
  * kernel (a 128-pixel tile's slab staged by the threads); 0 = mma.sync
- * (warp-level BF16 MMA). Results agree up to FP32 accumulation order. The
- * training forward takes the per-tile kernel under 1 and 2; inputs too wide
- * for a kernel's shared memory take the next one down. Process-wide. */
+ * (warp-level BF16 MMA). Results agree up to FP32 accumulation order. Training
+ * runs its forward pass and data gradients in the banded kernel under 1; under
+ * 2 its forward pass takes the per-tile kernel and its data gradients mma.sync.
+ * Inputs too wide for a kernel's shared memory take the next one down, and so
+ * do training batches whose padded activations pass 32 GB. Process-wide. */
 void bdis_set_net_variant(int tensor_path);
 int bdis_get_net_variant(void);
 

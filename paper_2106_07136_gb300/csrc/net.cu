@@ -17,11 +17,11 @@
 // Every convolution is an implicit GEMM (bf16 in, f32 accumulate): rows =
 // pixels, columns = output channels, K = 9 taps x input channels. The forward
 // convolutions run on the 5th-generation tensor cores (tcgen05, below) by
-// default, or on mma.sync.m16n8k16; training uses mma.sync. The data-gradient of a layer is the same kernel run on the
-// output gradient with transposed, tap-flipped weights and the previous
-// layer's ReLU mask fused into the store; the weight-gradient is a GEMM with
-// rows = output channels, columns = (tap, input channel), K = pixels, whose
-// blocks write partial sums that a second kernel adds in block order.
+// default, or on mma.sync.m16n8k16. The data-gradient of a layer is the same
+// kernel run on the output gradient with transposed, tap-flipped weights and
+// the previous layer's ReLU mask fused into the store; the weight-gradient is a
+// GEMM with rows = output channels, columns = (tap, input channel), K = pixels,
+// whose blocks write partial sums that a second kernel adds in a fixed order.
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(128) conv_tc_kernel(
 
 // ------------------------------------------- conv (tcgen05, banded inference)
 
-// The inference forward pass keeps every activation in a padded planar
+// The inference forward pass, and training, keep every activation in a padded planar
 // layout in global memory: each image is framed by kPad zero rows and
 // columns (kPad = the largest dilation, so every tap of a real pixel lands
 // inside its own frame), frames are numbered back to back, and each group of
@@ -491,12 +491,15 @@ __device__ __forceinline__ void *band_smem_base() {
 struct BandLayer {
   const __nv_bfloat16 *in, *wt;
   const float *bias;
-  void *out;      // kFwdRelu: padded planar bf16; kFwdLinearF32: dense float map
+  void *out;      // kFwdLinearF32: dense float map; else padded planar bf16
+  const __nv_bfloat16 *mask;  // kBwdDataMasked: the ReLU outputs (padded planar)
   int dil, BH, nsb;  // dilation, band rows, slab rows per channel plane
 };
 struct BandNet {
   BandLayer layer[6];
-  const float *L, *R;  // the level planes (R with element stride r_stride)
+  const float *L, *R;  // forward: the level planes (R with element stride r_stride)
+  const float *map, *label;  // backward: the forward map and its labels (NaN = none)
+  float *loss;               // backward: the loss, zero at launch
   int r_stride, H, W, count;
   int slab_bytes;      // per slab buffer (the largest layer's), two buffers
   unsigned *sync;      // grid barrier counter, zero at launch
@@ -537,13 +540,13 @@ __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target) {
 // One layer: the roles of the module comment over the layer's units. kg counts
 // the block's units over all layers (buffer = kg & 1, barrier phase = (kg >> 1)
 // & 1); on return every unit of the layer is written and its accumulators are
-// handed back. MODE kFwdRelu: out is a padded planar bf16 buffer of COUT
-// channels; kFwdLinearF32: out is the dense float map of channel 0.
+// handed back. MODE kFwdRelu, kBwdDataMasked: out is a padded planar bf16 buffer
+// of COUT channels (the latter zero where the layer's mask is not positive, no
+// bias); kFwdLinearF32: out is the dense float map of channel 0.
 template <int CIN, int COUT, int MODE>
 __device__ bool band_layer(const BandNet &net, const BandLayer &ly, const BandShared &sh,
                            float *sbias, long long &kg) {
   static_assert(CIN % 16 == 0 && (COUT == 16 || COUT == 32), "tile");
-  static_assert(MODE == kFwdRelu || MODE == kFwdLinearF32, "forward only");
   constexpr int KG = 9 * CIN / 8, NG = COUT / 8, CG = CIN / 8;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int H = net.H, W = net.W, count = net.count, dil = ly.dil, BH = ly.BH;
@@ -561,7 +564,7 @@ __device__ bool band_layer(const BandNet &net, const BandLayer &ly, const BandSh
     const uint4 v = *reinterpret_cast<const uint4 *>(ly.wt + (size_t)co * 9 * CIN + kgr * 8);
     *reinterpret_cast<uint4 *>(Bs + ((kgr * NG + co / 8) * 8 + co % 8) * 16) = v;
   }
-  if (tid < COUT) sbias[tid] = ly.bias[tid];
+  if (MODE != kBwdDataMasked && tid < COUT) sbias[tid] = ly.bias[tid];
   // weights: generic-proxy writes read by the tensor cores; the input: written
   // by other blocks before the grid barrier, read by this block's bulk copies
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -709,12 +712,28 @@ __device__ bool band_layer(const BandNet &net, const BandLayer &ly, const BandSh
         const int xp = m % Wp, x = xp - kPad;
         if (m < cnt && x >= 0 && x < W) {
           const long long q = q_s + m;
-          if constexpr (MODE == kFwdRelu) {
+          if constexpr (MODE != kFwdLinearF32) {
             uint32_t pk[COUT / 2];
-#pragma unroll
-            for (int c = 0; c < COUT; c += 2)
-              pk[c / 2] = pack_bf16(fmaxf(d[c] + bs[c], 0.f), fmaxf(d[c + 1] + bs[c + 1], 0.f));
             const long long plane_out = pp_plane(H, W, count) / 8;  // in 16-byte rows
+            if constexpr (MODE == kFwdRelu) {
+#pragma unroll
+              for (int c = 0; c < COUT; c += 2)
+                pk[c / 2] = pack_bf16(fmaxf(d[c] + bs[c], 0.f), fmaxf(d[c + 1] + bs[c + 1], 0.f));
+            } else {
+              const uint4 *mp = reinterpret_cast<const uint4 *>(ly.mask) + guard + q;
+#pragma unroll
+              for (int v = 0; v < COUT / 8; ++v) {
+                const uint4 m4 = __ldg(mp + v * plane_out);
+                const uint32_t mw[4] = {m4.x, m4.y, m4.z, m4.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const __nv_bfloat162 m = *reinterpret_cast<const __nv_bfloat162 *>(&mw[e]);
+                  const int c = 8 * v + 2 * e;
+                  pk[c / 2] = pack_bf16(__bfloat162float(m.x) > 0.f ? d[c] : 0.f,
+                                        __bfloat162float(m.y) > 0.f ? d[c + 1] : 0.f);
+                }
+              }
+            }
             uint4 *o = reinterpret_cast<uint4 *>(ly.out) + guard + q;
 #pragma unroll
             for (int v = 0; v < COUT / 8; ++v)
@@ -735,12 +754,25 @@ __device__ bool band_layer(const BandNet &net, const BandLayer &ly, const BandSh
   return __syncthreads_and(ok ? 1 : 0) != 0;
 }
 
-// The whole inference forward pass in one cooperative launch (one block per
-// SM): the input planes are packed into x0, then the six layers run in turn,
-// a grid barrier between steps (a layer reads the bands around its own, which
+// Huber (delta 1) loss of one pixel against its label (NaN = no label) over
+// the mean's 1 / n, and its gradient.
+__device__ __forceinline__ float huber_at(float z, float label, float inv_n, float &grad) {
+  grad = 0.f;
+  if (!isfinite(label)) return 0.f;
+  const float e = z - label, ae = fabsf(e);
+  grad = (ae <= 1.f ? e : copysignf(1.f, e)) * inv_n;
+  return ae <= 1.f ? 0.5f * e * e : ae - 0.5f;
+}
+
+// The whole forward pass (or, BACK, the loss and all data gradients) in one
+// cooperative launch (one block per SM): the input planes are packed into x0
+// (the loss gradient into the last layer's), then the layers run in turn, a
+// grid barrier between steps (a layer reads the bands around its own, which
 // other blocks wrote). Weights and bias are restaged per layer; the slabs,
-// barriers and tensor memory carry over.
-__global__ void __launch_bounds__(kBandThreads, 1) net_forward_kernel(const BandNet net) {
+// barriers and tensor memory carry over. BACK's layers are in their order of
+// execution, the last layer's data gradient first.
+template <bool BACK>
+__global__ void __launch_bounds__(kBandThreads, 1) net_chain_kernel(const BandNet net) {
   __shared__ __align__(8) uint64_t mb_full[2], mb_mma[2], mb_free[2];
   __shared__ uint32_t tmem_slot;
   __shared__ float sbias[32];
@@ -765,21 +797,33 @@ __global__ void __launch_bounds__(kBandThreads, 1) net_forward_kernel(const Band
                  "n"(2 * kBandCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
-  // x0: plane 0 = [(L - 128) / 64, (R - 128) / 64, 0 x 6] at every real pixel
-  // (plane 1 and the borders stay zero)
+  // x0: plane 0 = [(L - 128) / 64, (R - 128) / 64, 0 x 6] (BACK: the loss
+  // gradient, 0 x 7) at every real pixel (plane 1 and the borders stay zero)
   {
     const int H = net.H, W = net.W, Wp = W + 2 * kPad, Hp = H + 2 * kPad;
     const long long plane = (long long)H * W, total = plane * net.count;
     uint4 *x0 = reinterpret_cast<uint4 *>(const_cast<__nv_bfloat16 *>(net.layer[0].in));
+    const float inv_n = 1.f / (float)total;
+    float loss = 0.f;
     for (long long p = (long long)blockIdx.x * kBandThreads + tid; p < total;
          p += (long long)gridDim.x * kBandThreads) {
       const int b = (int)(p / plane);
       const int rem = (int)(p - (long long)b * plane);
       const int y = rem / W, x = rem - (rem / W) * W;
       const long long q = ((long long)b * Hp + y + kPad) * Wp + x + kPad;
-      const float l = (__ldg(net.L + p) - 128.f) * (1.f / 64.f);
-      const float r = (__ldg(net.R + p * net.r_stride) - 128.f) * (1.f / 64.f);
-      x0[pp_guard(W) + q] = make_uint4(pack_bf16(l, r), 0u, 0u, 0u);
+      if constexpr (BACK) {
+        float g;
+        loss += huber_at(__ldg(net.map + p), __ldg(net.label + p), inv_n, g);
+        x0[pp_guard(W) + q] = make_uint4(pack_bf16(g, 0.f), 0u, 0u, 0u);
+      } else {
+        const float l = (__ldg(net.L + p) - 128.f) * (1.f / 64.f);
+        const float r = (__ldg(net.R + p * net.r_stride) - 128.f) * (1.f / 64.f);
+        x0[pp_guard(W) + q] = make_uint4(pack_bf16(l, r), 0u, 0u, 0u);
+      }
+    }
+    if constexpr (BACK) {
+      for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+      if ((tid & 31) == 0) atomicAdd(net.loss, loss * inv_n);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -791,25 +835,33 @@ __global__ void __launch_bounds__(kBandThreads, 1) net_forward_kernel(const Band
   long long kg = 0;
   unsigned passed = 0;
   bool ok = grid_barrier(net.sync, ++passed * gridDim.x);
-  if (ok) ok = band_layer<16, 32, kFwdRelu>(net, net.layer[0], sh, sbias, kg);
+  constexpr int kMid = BACK ? kBwdDataMasked : kFwdRelu;
+  if (ok) ok = band_layer<16, 32, kMid>(net, net.layer[0], sh, sbias, kg);
   for (int l = 1; l < 5 && ok; ++l) {
     ok = grid_barrier(net.sync, ++passed * gridDim.x);
-    if (ok) ok = band_layer<32, 32, kFwdRelu>(net, net.layer[l], sh, sbias, kg);
+    if (ok) ok = band_layer<32, 32, kMid>(net, net.layer[l], sh, sbias, kg);
   }
-  if (ok) ok = grid_barrier(net.sync, ++passed * gridDim.x);
-  if (ok) ok = band_layer<32, 16, kFwdLinearF32>(net, net.layer[5], sh, sbias, kg);
+  if constexpr (!BACK) {
+    if (ok) ok = grid_barrier(net.sync, ++passed * gridDim.x);
+    if (ok) ok = band_layer<32, 16, kFwdLinearF32>(net, net.layer[5], sh, sbias, kg);
+  }
   if (!ok) {
-    // a wait ran out (ok is uniform over the block): record it, and mark this
-    // block's bands of the map as missing (NaN), whatever was written there
+    // a wait ran out (ok is uniform over the block): record it, and mark the
+    // loss, or this block's bands of the map, as missing (NaN), whatever was
+    // written there
     if (tid == 0) atomicOr(net.fault, 1);
-    const BandLayer &ly = net.layer[5];
-    const int H = net.H, W = net.W, nb = (H + ly.BH - 1) / ly.BH;
-    const long long units = (long long)net.count * nb;
-    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
-      const int b = (int)(u / nb), j = (int)(u - (long long)b * nb);
-      const int n = min(ly.BH, H - j * ly.BH) * W;
-      float *o = reinterpret_cast<float *>(ly.out) + ((long long)b * H + j * ly.BH) * W;
-      for (int i = tid; i < n; i += kBandThreads) o[i] = __int_as_float(0x7fc00000);
+    if constexpr (BACK) {
+      if (tid == 0) atomicExch(net.loss, __int_as_float(0x7fc00000));
+    } else {
+      const BandLayer &ly = net.layer[5];
+      const int H = net.H, W = net.W, nb = (H + ly.BH - 1) / ly.BH;
+      const long long units = (long long)net.count * nb;
+      for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+        const int b = (int)(u / nb), j = (int)(u - (long long)b * nb);
+        const int n = min(ly.BH, H - j * ly.BH) * W;
+        float *o = reinterpret_cast<float *>(ly.out) + ((long long)b * H + j * ly.BH) * W;
+        for (int i = tid; i < n; i += kBandThreads) o[i] = __int_as_float(0x7fc00000);
+      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -827,22 +879,24 @@ __global__ void __launch_bounds__(kBandThreads, 1) net_forward_kernel(const Band
 // ci), K = pixels: 32 rows at most, which tcgen05's M of 64 or 128 would leave
 // half empty, and both operands pixel-major).
 //
-// Pixels are numbered in frames of (H + dil) x (W + dil) positions per image,
-// zero past the image: the zeros right of a row and below an image are also
-// those left of the next row and above the next image, so a tap is a constant
-// shift. A block takes tiles of 128 positions of one layer. Per tile it stages
-// G once and X as three segments of 128 + 2 dil positions (one per kernel
-// row, whatever the image width), two tiles in flight. ldmatrix.trans turns
-// the pixel-major rows into both operands' fragments; rows are swizzled so that
-// eight consecutive ones fall in distinct banks. A warp owns 8 input channels
-// (the first layer, with 2, is split over the warps by pixels instead) and all
-// nine taps; a block writes its totals to a partial buffer of its own, which
-// reduce_grad_kernel adds in a fixed order: no atomics, the same gradient every
-// time. Six launches that staged nine shifted copies of X word by word took
-// 500 us per 64 images of 40x30, of a gradient call's 780; it is now 310.
+// Pixels are numbered so that a tap is a constant shift: for activations in the
+// banded kernel's padded planar layout (PLANAR) by their positions there, the
+// padded rows of an image after one another; for NHWC ones (images too wide for
+// the banded kernel) in frames of (H + dil) x (W + dil) positions, zero past the
+// image. A block takes tiles of 128 positions of one layer. Per tile it stages
+// G once and X as three segments of 128 + 2 dil positions (one per kernel row,
+// whatever the image width), a plane of 16-byte rows per 8 channels, two tiles
+// in flight: from the planar layout by one bulk copy per plane and segment.
+// ldmatrix.trans turns the pixel-major rows into both operands' fragments (eight
+// rows are 128 consecutive bytes: no bank conflicts). A warp owns 8 input
+// channels (the first layer, with 2, is split over the warps by pixels instead)
+// and all nine taps; a block writes its totals to a partial buffer of its own,
+// which reduce_grad_kernel adds in a fixed order: no atomics, the same gradient
+// every time.
 constexpr int kWgTile = 128;
 constexpr int kWgRows = kWgTile + 2 * 4;  // rows of a segment at the largest dilation
-constexpr int kWgStage = (3 * kWgRows + kWgTile) * 64;  // bytes of one staged tile (X, then G)
+constexpr int kWgX = 3 * kWgRows * 16, kWgG = kWgTile * 16;  // bytes of a staged plane
+constexpr int kWgStage = 4 * (kWgX + kWgG);  // bytes of one staged tile (X, then G)
 constexpr int kWgSmem = 2 * kWgStage, kWgPerSm = 3;  // 3 x 67 KB per SM
 constexpr int kPart = 32 * 9 * 32 + 32;  // floats of one block's partial: dW, then db
 
@@ -854,6 +908,7 @@ struct WgradArgs {
   WgradLayer layer[kLayers];
   int H, W, count;
   float *part;
+  int *fault;
 };
 
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
@@ -862,30 +917,28 @@ __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
                : "r"(addr));
 }
 
-// byte offset of 16-byte chunk c of a row of C chunks (1 or 4)
-template <int C>
-__device__ __forceinline__ uint32_t wg_chunk(int row, int c) {
-  static_assert(C == 1 || C == 4, "chunks per row");
-  return C == 1 ? row * 16 : row * 64 + ((c ^ ((row >> 1) & 3)) << 4);
-}
-
 // One layer's tiles t = rank, rank + ranks, ... XS, GS: channels stored per
-// pixel; XC, GC: 16-byte chunks (8 channels) of them used; CO: real output
-// channels; CI: real input channels.
-template <int XS, int XC, int GS, int GC>
-__device__ __forceinline__ void wgrad_layer(const WgradArgs &args, const WgradLayer &ly,
-                                            uint8_t *smem, float *part) {
+// pixel (NHWC); XC, GC: planes of 8 channels used. False if a bounded wait for
+// the copies ran out.
+template <bool PLANAR, int XS, int XC, int GS, int GC>
+__device__ __forceinline__ bool wgrad_layer(const WgradArgs &args, const WgradLayer &ly,
+                                            uint8_t *smem, uint32_t mbar, float *part) {
   constexpr int MT = (GC + 1) / 2;       // 16-channel m-tiles
   constexpr bool SPLIT = XC < 4;         // warps share the pixels, not the channels
   static_assert(XC == 1 || XC == 4, "one warp per 8 input channels, or one group");
   constexpr int CIW = XC * 8;            // input channels of the partial
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int H = args.H, W = args.W, dil = ly.dil, Wp = W + dil, Hp = H + dil;
-  const long long frame = (long long)Hp * Wp, total = frame * args.count;
-  const long long tiles = (total + kWgTile - 1) / kWgTile;
+  const int H = args.H, W = args.W, dil = ly.dil;
+  const int Wp = W + (PLANAR ? 2 * kPad : dil), Hp = H + (PLANAR ? 2 * kPad : dil);
+  const long long frame = (long long)Hp * Wp;
+  // PLANAR: tiles of each image's rows (H Wp positions); else of all positions
+  const int per_image = (H * Wp + kWgTile - 1) / kWgTile;
+  const long long total = frame * args.count;
+  const long long tiles = PLANAR ? (long long)per_image * args.count : (total + kWgTile - 1) / kWgTile;
+  const long long plane = PLANAR ? pp_plane(H, W, args.count) / 8 : 0, guard = pp_guard(W);
   const int seg = kWgTile + 2 * dil, rank = (int)blockIdx.x - ly.first;
   const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
-  const uint32_t goff = 3 * kWgRows * 64;
+  constexpr uint32_t goff = XC * kWgX;
   auto pixel = [&](long long q) -> long long {
     if (q < 0 || q >= total) return -1;
     int b, rem;
@@ -901,39 +954,63 @@ __device__ __forceinline__ void wgrad_layer(const WgradArgs &args, const WgradLa
   };
   auto stage = [&](long long tile, int buf) {
     const uint32_t base = s0 + buf * kWgStage;
-    for (int i = tid; i < 3 * seg + kWgTile; i += 128) {
-      const bool isx = i < 3 * seg;
-      const int ty = i / seg, row = isx ? i - ty * seg : i - 3 * seg;
-      const long long q = tile * kWgTile + (isx ? (long long)(ty - 1) * dil * Wp - dil : 0) + row;
-      const long long p = pixel(q);
-      const int ok = p >= 0 ? 16 : 0;
-      if (isx) {
+    if constexpr (PLANAR) {
+      const int b = (int)(tile / per_image), i = (int)(tile - (long long)b * per_image) * kWgTile;
+      const int n = min(kWgTile, H * Wp - i);  // positions of the tile; G past them is zero
+      const long long q = guard + b * frame + (long long)kPad * Wp + i;
+      if (n < kWgTile && warp != 0)
+        for (int r = n + tid - 32; r < kWgTile; r += 96)
 #pragma unroll
+          for (int c = 0; c < GC; ++c)
+            *reinterpret_cast<uint4 *>(smem + buf * kWgStage + goff + c * kWgG + r * 16) =
+                make_uint4(0u, 0u, 0u, 0u);
+      if (tid == 0) {
+        // the buffer's last reads (ldmatrix) come before these writes
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        mbar_expect_tx(mbar + 8 * buf, (uint32_t)(XC * 3 * seg + GC * n) * 16u);
         for (int c = 0; c < XC; ++c)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
-                           base + wg_chunk<XC>(i, c)),
-                       "l"(ly.X + (p >= 0 ? p * XS + c * 8 : 0)), "r"(ok));
-      } else {
-#pragma unroll
+          for (int ty = 0; ty < 3; ++ty)
+            bulk_load(base + c * kWgX + ty * seg * 16,
+                      ly.X + (c * plane + q + (long long)(ty - 1) * dil * Wp - dil) * 8,
+                      (uint32_t)seg * 16u, mbar + 8 * buf);
         for (int c = 0; c < GC; ++c)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
-                           base + goff + wg_chunk<GC>(row, c)),
-                       "l"(ly.G + (p >= 0 ? p * GS + c * 8 : 0)), "r"(ok));
+          bulk_load(base + goff + c * kWgG, ly.G + (c * plane + q) * 8, (uint32_t)n * 16u,
+                    mbar + 8 * buf);
       }
+    } else {
+      for (int i = tid; i < 3 * seg + kWgTile; i += 128) {
+        const bool isx = i < 3 * seg;
+        const int ty = i / seg, row = isx ? i - ty * seg : i - 3 * seg;
+        const long long q = tile * kWgTile + (isx ? (long long)(ty - 1) * dil * Wp - dil : 0) + row;
+        const long long p = pixel(q);
+        const int ok = p >= 0 ? 16 : 0;
+        if (isx) {
+#pragma unroll
+          for (int c = 0; c < XC; ++c)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                             base + c * kWgX + i * 16),
+                         "l"(ly.X + (p >= 0 ? p * XS + c * 8 : 0)), "r"(ok));
+        } else {
+#pragma unroll
+          for (int c = 0; c < GC; ++c)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                             base + goff + c * kWgG + row * 16),
+                         "l"(ly.G + (p >= 0 ? p * GS + c * 8 : 0)), "r"(ok));
+        }
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
-  // the lane's ldmatrix row offsets: X rows of tap t for pixels 0 .. 31 of the
-  // tile, G rows for pixels 0 .. 15 (both advance by whole multiples of 32 rows,
-  // which leaves the swizzle as it is)
+  // the lane's ldmatrix rows: X rows of tap t for pixels 0 .. 31 of the tile, G
+  // rows for pixels 0 .. 15
   uint32_t xo[9], go[MT];
 #pragma unroll
   for (int t = 0; t < 9; ++t)
-    xo[t] = wg_chunk<XC>((t / 3) * seg + dil + (t % 3 - 1) * dil + lane, SPLIT ? 0 : warp);
+    xo[t] = (SPLIT ? 0 : warp) * kWgX + ((t / 3) * seg + (t % 3) * dil + lane) * 16;
 #pragma unroll
   for (int m = 0; m < MT; ++m) {
-    const int mat = lane >> 3, chunk = m * 2 + (mat & 1);
-    go[m] = goff + wg_chunk<GC>((mat >> 1) * 8 + (lane & 7), GC == 1 ? 0 : chunk);
+    const int mat = lane >> 3, c = GC == 1 ? 0 : m * 2 + (mat & 1);
+    go[m] = goff + c * kWgG + ((mat >> 1) * 8 + (lane & 7)) * 16;
   }
   float acc[MT][9][4], adb[MT][4];
 #pragma unroll
@@ -945,9 +1022,21 @@ __device__ __forceinline__ void wgrad_layer(const WgradArgs &args, const WgradLa
   const uint32_t ones[2] = {0x3f803f80u, 0x3f803f80u};
   if (rank < tiles) stage(rank, 0);
   int buf = 0;
+  uint32_t phases = 0u;  // bit b: the parity that buffer b's copies complete next
   for (long long tile = rank; tile < tiles; tile += ly.blocks, buf ^= 1) {
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-    __syncthreads();  // tile staged; the other buffer is read no more
+    bool ok = true;
+    if constexpr (PLANAR) {
+      ok = mbar_wait(mbar + 8 * buf, (phases >> buf) & 1u);
+    } else {
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+    }
+    // tile staged; the other buffer is read no more (and, after a wait that ran
+    // out, no copy but this one is in flight: give it one more wait)
+    if (!__syncthreads_and(ok)) {
+      mbar_wait(mbar + 8 * buf, (phases >> buf) & 1u);
+      return false;
+    }
+    phases ^= 1u << buf;
     if (tile + ly.blocks < tiles) stage(tile + ly.blocks, buf ^ 1);
     const uint32_t base = s0 + buf * kWgStage;
 #pragma unroll 1
@@ -957,7 +1046,7 @@ __device__ __forceinline__ void wgrad_layer(const WgradArgs &args, const WgradLa
       for (int m = 0; m < MT; ++m)
 #pragma unroll
         for (int ks = 0; ks < 2; ++ks) {
-          ldsm4t(ga[m][ks], base + go[m] + (k32 * 32 + ks * 16) * (GC * 16));
+          ldsm4t(ga[m][ks], base + go[m] + (k32 * 32 + ks * 16) * 16);
           if (GC == 1) ga[m][ks][1] = ga[m][ks][3] = 0u;  // channels 8 .. 15 do not exist
         }
       // a kernel row's three taps at a time: 3 MT independent MMAs before the
@@ -967,7 +1056,7 @@ __device__ __forceinline__ void wgrad_layer(const WgradArgs &args, const WgradLa
         uint32_t xb[3][4];
 #pragma unroll
         for (int tx = 0; tx < 3; ++tx)
-          ldsm4t(xb[tx], base + xo[ty * 3 + tx] + k32 * 32 * (XC * 16));
+          ldsm4t(xb[tx], base + xo[ty * 3 + tx] + k32 * 32 * 16);
 #pragma unroll
         for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
@@ -1017,20 +1106,37 @@ __device__ __forceinline__ void wgrad_layer(const WgradArgs &args, const WgradLa
     for (int i = tid; i < GC * 8 * 9 * CIW; i += 128) part[i] = dst[i];
     if (tid < GC * 8) part[kPart - 32 + tid] = dst[kPart - 32 + tid];
   }
+  return true;
 }
 
+template <bool PLANAR>
 __global__ void __launch_bounds__(128, kWgPerSm) conv_wgrad_kernel(const WgradArgs args) {
   extern __shared__ __align__(128) uint8_t wg_smem[];
+  __shared__ __align__(8) uint64_t mbars[2];
+  const uint32_t mbar = (uint32_t)__cvta_generic_to_shared(mbars);
+  if (threadIdx.x == 0) {
+    mbar_init(mbar, 1);
+    mbar_init(mbar + 8, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncthreads();
   bdis::pdl_enter();
+  // the activations, written by other kernels' plain stores, are read by copies
+  asm volatile("fence.proxy.async.global;\n" ::: "memory");
   int l = 0;
   while (l + 1 < kLayers && (int)blockIdx.x >= args.layer[l + 1].first) ++l;
   float *part = args.part + (long long)blockIdx.x * kPart;
+  bool ok;
   if (l == 0)
-    wgrad_layer<16, 1, 32, 4>(args, args.layer[0], wg_smem, part);
+    ok = wgrad_layer<PLANAR, 16, 1, 32, 4>(args, args.layer[0], wg_smem, mbar, part);
   else if (l == 5)
-    wgrad_layer<32, 4, 16, 1>(args, args.layer[5], wg_smem, part);
+    ok = wgrad_layer<PLANAR, 32, 4, 16, 1>(args, args.layer[5], wg_smem, mbar, part);
   else
-    wgrad_layer<32, 4, 32, 4>(args, args.layer[l], wg_smem, part);
+    ok = wgrad_layer<PLANAR, 32, 4, 32, 4>(args, args.layer[l], wg_smem, mbar, part);
+  if (!ok) {  // reported by bdis_net_status; the gradient is not a number
+    if (threadIdx.x == 0) atomicOr(args.fault, 1);
+    for (int i = threadIdx.x; i < kPart; i += 128) part[i] = __int_as_float(0x7fc00000);
+  }
 }
 
 struct LayerBlocks {
@@ -1086,13 +1192,7 @@ __global__ void loss_kernel(const float *__restrict__ z6, const float *__restric
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   float l = 0.f, gr = 0.f;
   if (p < total) {
-    const float y = label[p];
-    if (isfinite(y)) {
-      const float e = z6[p * 16] - y;
-      const float ae = fabsf(e);
-      l = ae <= 1.f ? 0.5f * e * e : ae - 0.5f;
-      gr = (ae <= 1.f ? e : copysignf(1.f, e)) * inv_n;
-    }
+    l = huber_at(z6[p * 16], label[p], inv_n, gr);
     uint4 *dst = reinterpret_cast<uint4 *>(g6 + p * 16);
     dst[0] = make_uint4(pack_bf16(gr, 0.f), 0u, 0u, 0u);
     dst[1] = make_uint4(0u, 0u, 0u, 0u);
@@ -1166,9 +1266,13 @@ struct bdis_net {
   // device word set when a forward kernel's bounded wait ran out
   int *fault = nullptr;
   unsigned *sync = nullptr;  // grid barrier counter of the fused inference kernel
-  // inference activations in the padded planar layout, for pp_h x pp_w x pp_count
-  __nv_bfloat16 *x0pp = nullptr, *app[5] = {};
-  int pp_h = 0, pp_w = 0, pp_count = 0;
+  // activations in the padded planar layout for count h x w images: of
+  // inference, and of training (with the gradients of the layers' outputs)
+  struct Planar {
+    __nv_bfloat16 *x0 = nullptr, *a[5] = {}, *g[5] = {}, *g6 = nullptr;
+    float *map = nullptr;  // training: the forward map
+    int h = 0, w = 0, count = 0;
+  } infer, train;
 };
 
 namespace {
@@ -1179,51 +1283,71 @@ void net_free_acts(bdis_net *n) {
   for (auto &p : n->gact) cudaFree(p);
   cudaFree(n->g6);
   cudaFree(n->z6);
-  cudaFree(n->part);
   n->x0 = nullptr;
   for (auto &p : n->a) p = nullptr;
   for (auto &p : n->gact) p = nullptr;
   n->g6 = nullptr;
   n->z6 = nullptr;
-  n->part = nullptr;
   n->cap = 0;
 }
 
-void net_free_pp(bdis_net *n) {
-  cudaFree(n->x0pp);
-  for (auto &p : n->app) cudaFree(p);
-  n->x0pp = nullptr;
-  for (auto &p : n->app) p = nullptr;
-  n->pp_h = n->pp_w = n->pp_count = 0;
+void net_free_planar(bdis_net::Planar &p) {
+  cudaFree(p.x0);
+  for (auto &q : p.a) cudaFree(q);
+  for (auto &q : p.g) cudaFree(q);
+  cudaFree(p.g6);
+  cudaFree(p.map);
+  p = bdis_net::Planar();
 }
 
-// Padded planar activations of the inference pass for count h x w images,
-// zeroed (borders and guards stay zero: only real pixels are ever written).
-bdis_status net_reserve_pp(bdis_net *n, int h, int w, int count, cudaStream_t st) {
-  if (n->pp_h == h && n->pp_w == w && n->pp_count == count) return BDIS_OK;
-  net_free_pp(n);
+// Padded planar activations for count h x w images (with `train`, also the
+// gradients), zeroed (borders and guards stay zero: only real pixels are ever
+// written).
+bdis_status net_reserve_planar(bdis_net::Planar &p, int h, int w, int count, bool train,
+                               cudaStream_t st) {
+  if (p.h == h && p.w == w && p.count == count) return BDIS_OK;
+  net_free_planar(p);
   const size_t plane = (size_t)pp_plane(h, w, count) * sizeof(__nv_bfloat16);
-  cudaError_t e = bdis::device_alloc((void **)&n->x0pp, 2 * plane);
-  for (auto &p : n->app)
-    if (e == cudaSuccess) e = bdis::device_alloc((void **)&p, 4 * plane);
-  if (e == cudaSuccess) e = cudaMemsetAsync(n->x0pp, 0, 2 * plane, st);
-  for (auto &p : n->app)
-    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, 4 * plane, st);
+  cudaError_t e = cudaSuccess;
+  auto take = [&](__nv_bfloat16 *&q, int planes) {
+    if (e == cudaSuccess) e = bdis::device_alloc((void **)&q, planes * plane);
+    if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, planes * plane, st);
+  };
+  take(p.x0, 2);
+  for (auto &q : p.a) take(q, 4);
+  if (train) {
+    for (auto &q : p.g) take(q, 4);
+    take(p.g6, 2);
+    if (e == cudaSuccess)
+      e = bdis::device_alloc((void **)&p.map, sizeof(float) * (size_t)h * w * count);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
-    net_free_pp(n);
+    net_free_planar(p);
     return e == cudaErrorMemoryAllocation ? BDIS_E_NOMEM : bdis::record_cuda(e);
   }
-  n->pp_h = h;
-  n->pp_w = w;
-  n->pp_count = count;
+  p.h = h;
+  p.w = w;
+  p.count = count;
   return BDIS_OK;
 }
 
-// Activations for `pixels` pixels; with `train`, also the gradients of every
-// layer's output and the weight gradient's partial sums.
+// The weight gradient's partial sums.
+bdis_status net_reserve_part(bdis_net *n) {
+  if (n->part) return BDIS_OK;
+  n->part_blocks = kWgPerSm * bdis::device_sms() + kLayers;
+  if (bdis::device_alloc((void **)&n->part, sizeof(float) * kPart * n->part_blocks) != cudaSuccess) {
+    cudaGetLastError();
+    n->part = nullptr;
+    return BDIS_E_NOMEM;
+  }
+  return BDIS_OK;
+}
+
+// NHWC activations for `pixels` pixels; with `train`, also the gradients of
+// every layer's output.
 bdis_status net_reserve(bdis_net *n, long long pixels, bool train) {
-  if (pixels <= n->cap && (!train || n->part)) return BDIS_OK;
+  if (pixels <= n->cap && (!train || n->gact[0])) return BDIS_OK;
   pixels = std::max(pixels, n->cap);
   net_free_acts(n);
   cudaError_t e = cudaSuccess;
@@ -1232,11 +1356,8 @@ bdis_status net_reserve(bdis_net *n, long long pixels, bool train) {
   };
   alloc((void **)&n->x0, pixels * 16 * 2);
   for (auto &p : n->a) alloc((void **)&p, pixels * 32 * 2);
-  if (train) {
+  if (train)
     for (auto &p : n->gact) alloc((void **)&p, pixels * 32 * 2);
-    n->part_blocks = kWgPerSm * bdis::device_sms() + kLayers;
-    alloc((void **)&n->part, sizeof(float) * kPart * n->part_blocks);
-  }
   alloc((void **)&n->g6, pixels * 16 * 2);
   alloc((void **)&n->z6, pixels * 16 * 4);
   if (e != cudaSuccess) {
@@ -1345,64 +1466,65 @@ int band_rows(int dil, int H, int W, int *nsb_out) {
   return 0;
 }
 
-// The inference forward pass as one cooperative launch of net_forward_kernel:
-// level planes in, the proposal (channel 0 of the last layer) written straight
-// to `out`. Returns false, having launched nothing, when the images are too
-// wide for it or the device cannot run the grid cooperatively.
-bool forward_pp(bdis_net *n, const float *L3, const float *R3, int r_stride, int H, int W,
-                int count, float *out, cudaStream_t st) {
-  if (g_net_tc != 1) return false;
-  BandNet net{};
-  int nsb[6], bh[6];
-  bh[0] = band_rows<16, 32>(kDil[0], H, W, &nsb[0]);
-  for (int l = 1; l < 5; ++l) bh[l] = band_rows<32, 32>(kDil[l], H, W, &nsb[l]);
-  bh[5] = band_rows<32, 16>(kDil[5], H, W, &nsb[5]);
+// Whether images of this size fit the banded kernel (its slabs, every layer).
+bool band_fits(int H, int W) {
+  int nsb = 0;
+  return band_rows<32, 32>(4, H, W, &nsb) && band_rows<16, 32>(1, H, W, &nsb) &&
+         band_rows<32, 16>(1, H, W, &nsb);
+}
+
+// One cooperative launch of net_chain_kernel<BACK> over `layers` layers with
+// their buffers filled in (dilation included): picks the band heights. Returns
+// false, having launched nothing, when the images are too wide for it or the
+// device cannot run the grid cooperatively.
+template <bool BACK>
+bool launch_chain(bdis_net *n, BandNet &net, int H, int W, int count, cudaStream_t st) {
+  const int layers = BACK ? 5 : 6;
+  int nsb[6] = {}, bh[6] = {};
+  for (int l = 0; l < layers; ++l)
+    bh[l] = l == 0   ? band_rows<16, 32>(net.layer[l].dil, H, W, &nsb[l])
+            : l == 5 ? band_rows<32, 16>(net.layer[l].dil, H, W, &nsb[l])
+                     : band_rows<32, 32>(net.layer[l].dil, H, W, &nsb[l]);
   // Band heights. Small batches: bands of fewer rows, so that a layer's
   // bands spread over the SMs (a single 40x30 image would otherwise be two
   // bands on two SMs, the rest waiting at the grid barriers). Then the bands
   // of an image are made equal (30 rows: 15 + 15, not 21 + 9): blocks take
   // bands round robin, and unequal bands would give every other block all
-  // the tall ones. A proposal does not depend on the band height: each
+  // the tall ones. A result does not depend on the band height: each
   // position's MMAs and epilogue are the same.
   const int per_image = (g_sms + count - 1) / count;  // bands wanted per image
   const int want = std::max(1, (H + per_image - 1) / per_image);
   int slab = 0;
-  for (int l = 0; l < 6; ++l) {
+  // one block per SM, or one per band where a layer has fewer bands (a
+  // single image): fewer blocks meet at each grid barrier and restage the
+  // weights
+  long long units = 1;
+  for (int l = 0; l < layers; ++l) {
     if (!bh[l]) return false;
     const int nb = (H + std::min(want, bh[l]) - 1) / std::min(want, bh[l]);
     const int even = (H + nb - 1) / nb;  // <= bh[l]: the limits still hold
     if (even < bh[l]) {
-      const int Wp = W + 2 * kPad, soff = kDil[l] * Wp + kDil[l];
+      const int Wp = W + 2 * kPad, soff = net.layer[l].dil * Wp + net.layer[l].dil;
       bh[l] = even;
       nsb[l] = (even * Wp + 127) / 128 * 128 + 2 * soff;
     }
-    slab = std::max(slab, (kCinP[l] / 8) * nsb[l] * 16);
+    net.layer[l].BH = bh[l];
+    net.layer[l].nsb = nsb[l];
+    slab = std::max(slab, (l == 0 ? 2 : 4) * nsb[l] * 16);
+    units = std::max(units, (long long)count * ((H + bh[l] - 1) / bh[l]));
   }
   const int smem = 2 * slab + kBandWeightsMax;
   static uint64_t attr_set = 0;  // bit d: the shared-memory limit is set on device d
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 64 || !(attr_set >> dev & 1u)) {
-    if (cudaFuncSetAttribute(net_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(net_chain_kernel<BACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kBandSmem) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
     if (dev < 64) attr_set |= 1ull << dev;
   }
-  const __nv_bfloat16 *ins[6] = {n->x0pp, n->app[0], n->app[1], n->app[2], n->app[3], n->app[4]};
-  for (int l = 0; l < 6; ++l) {
-    net.layer[l].in = ins[l];
-    net.layer[l].wt = n->wf[l];
-    net.layer[l].bias = n->bias[l];
-    net.layer[l].out = l < 5 ? (void *)n->app[l] : (void *)out;
-    net.layer[l].dil = kDil[l];
-    net.layer[l].BH = bh[l];
-    net.layer[l].nsb = nsb[l];
-  }
-  net.L = L3;
-  net.R = R3;
-  net.r_stride = r_stride;
   net.H = H;
   net.W = W;
   net.count = count;
@@ -1413,20 +1535,55 @@ bool forward_pp(bdis_net *n, const float *L3, const float *R3, int r_stride, int
     cudaGetLastError();
     return false;
   }
-  // one block per SM, or one per band where a layer has fewer bands (a
-  // single image): fewer blocks meet at each grid barrier and restage the
-  // weights
-  long long units = 1;
-  for (int l = 0; l < 6; ++l)
-    units = std::max(units, (long long)count * ((H + bh[l] - 1) / bh[l]));
   const unsigned grid = (unsigned)std::min<long long>(g_sms, units);
   void *args[] = {&net};
-  if (cudaLaunchCooperativeKernel((const void *)net_forward_kernel, dim3(grid),
+  if (cudaLaunchCooperativeKernel((const void *)net_chain_kernel<BACK>, dim3(grid),
                                   dim3(kBandThreads), args, (size_t)smem, st) != cudaSuccess) {
     cudaGetLastError();  // not sticky: the per-tile kernels run instead
     return false;
   }
   return true;
+}
+
+// The forward pass as one cooperative launch: level planes in, the proposal
+// (channel 0 of the last layer) written straight to `out`.
+bool forward_planar(bdis_net *n, const bdis_net::Planar &p, const float *L3, const float *R3,
+                    int r_stride, int H, int W, int count, float *out, cudaStream_t st) {
+  BandNet net{};
+  for (int l = 0; l < 6; ++l) {
+    net.layer[l].in = l ? p.a[l - 1] : p.x0;
+    net.layer[l].wt = n->wf[l];
+    net.layer[l].bias = n->bias[l];
+    net.layer[l].out = l < 5 ? (void *)p.a[l] : (void *)out;
+    net.layer[l].dil = kDil[l];
+  }
+  net.L = L3;
+  net.R = R3;
+  net.r_stride = r_stride;
+  return launch_chain<false>(n, net, H, W, count, st);
+}
+
+// The loss and every layer's data gradient as one cooperative launch, on the
+// activations that forward_planar left.
+bool backward_planar(bdis_net *n, const bdis_net::Planar &p, const float *label, int H, int W,
+                     int count, cudaStream_t st) {
+  BandNet net{};
+  for (int i = 0; i < 5; ++i) {  // the gradient of layer l's output becomes that of its input
+    const int l = 5 - i;
+    net.layer[i].in = l == 5 ? p.g6 : p.g[l];
+    net.layer[i].wt = n->wb[l];
+    net.layer[i].mask = p.a[l - 1];
+    net.layer[i].out = p.g[l - 1];
+    net.layer[i].dil = kDil[l];
+  }
+  net.map = p.map;
+  net.label = label;
+  net.loss = n->loss;
+  if (cudaMemsetAsync(n->loss, 0, sizeof(float), st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return launch_chain<true>(n, net, H, W, count, st);
 }
 
 cudaError_t forward(bdis_net *n, const float *L3, const float *R3, int r_stride, int H, int W,
@@ -1442,25 +1599,21 @@ cudaError_t forward(bdis_net *n, const float *L3, const float *R3, int r_stride,
   return cudaGetLastError();
 }
 
-// Backward through all layers: the data gradients, layer by layer, then every
-// layer's weight gradient in one launch and the sum of its partials.
-cudaError_t backward(bdis_net *n, int H, int W, long long total, cudaStream_t st) {
-  // g5 = (W6^T g6) * relu'(a5)
-  conv<16, 32, kBwdDataMasked>(n->g6, n->wb[5], nullptr, kDil[5], H, W, total, n->a[4],
-                               n->gact[4], n->fault, st);
-  for (int l = 4; l >= 1; --l)
-    conv<32, 32, kBwdDataMasked>(n->gact[l], n->wb[l], nullptr, kDil[l], H, W, total,
-                                 n->a[l - 1], n->gact[l - 1], n->fault, st);
-  // Blocks per layer: as many in all as run at once, in proportion to the layers' work (a
-  // tile of the first or last layer is a fraction of a middle one's)
+// Every layer's weight gradient in one launch, on planar activations or (p
+// null) NHWC ones, and the sum of its partials.
+cudaError_t weight_gradients(bdis_net *n, const bdis_net::Planar *p, int H, int W, int count,
+                             cudaStream_t st) {
+  // Blocks per layer: as many in all as run at once, in proportion to the
+  // layers' work (a tile of the first or last layer is a fraction of a middle
+  // one's)
   static const double kCost[kLayers] = {0.4, 1, 1, 1, 1, 0.6};
   WgradArgs wa{};
   LayerBlocks lb{};
-  const int count = (int)(total / ((long long)H * W));
   long long tiles[kLayers];
   double work = 0;
   for (int l = 0; l < kLayers; ++l) {
-    tiles[l] = ((long long)(H + kDil[l]) * (W + kDil[l]) * count + kWgTile - 1) / kWgTile;
+    tiles[l] = p ? (long long)((H * (W + 2 * kPad) + kWgTile - 1) / kWgTile) * count
+                 : ((long long)(H + kDil[l]) * (W + kDil[l]) * count + kWgTile - 1) / kWgTile;
     work += tiles[l] * kCost[l];
   }
   int blocks = 0;
@@ -1469,28 +1622,43 @@ cudaError_t backward(bdis_net *n, int H, int W, long long total, cudaStream_t st
     lb.first[l] = blocks;
     lb.blocks[l] = (int)std::max(1ll, std::min(tiles[l], (long long)share));
     blocks += lb.blocks[l];
-    wa.layer[l] = {l ? n->a[l - 1] : n->x0, l < 5 ? n->gact[l] : n->g6, kDil[l], lb.first[l],
-                   lb.blocks[l]};
+    wa.layer[l] = {p ? (l ? p->a[l - 1] : p->x0) : (l ? n->a[l - 1] : n->x0),
+                   p ? (l < 5 ? p->g[l] : p->g6) : (l < 5 ? n->gact[l] : n->g6), kDil[l],
+                   lb.first[l], lb.blocks[l]};
   }
   wa.H = H;
   wa.W = W;
   wa.count = count;
   wa.part = n->part;
-  cudaError_t e = cudaFuncSetAttribute(conv_wgrad_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
+  wa.fault = n->fault;
+  auto kernel = p ? conv_wgrad_kernel<true> : conv_wgrad_kernel<false>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
   if (e == cudaSuccess)
-    e = bdis::launch_maybe_overlapped(conv_wgrad_kernel, dim3((unsigned)blocks), dim3(128),
-                                      (size_t)kWgSmem, st, wa);
+    e = bdis::launch_maybe_overlapped(kernel, dim3((unsigned)blocks), dim3(128), (size_t)kWgSmem,
+                                      st, wa);
   if (e == cudaSuccess)
     e = bdis::launch_maybe_overlapped(reduce_grad_kernel, dim3(nblocks(kMasterCount, 32)),
                                       dim3(256), 0, st, (const float *)n->part, lb, n->grad);
   return e;
 }
 
+// The data gradients of NHWC activations, layer by layer.
+void data_gradients(bdis_net *n, int H, int W, long long total, cudaStream_t st) {
+  // g5 = (W6^T g6) * relu'(a5)
+  conv<16, 32, kBwdDataMasked>(n->g6, n->wb[5], nullptr, kDil[5], H, W, total, n->a[4],
+                               n->gact[4], n->fault, st);
+  for (int l = 4; l >= 1; --l)
+    conv<32, 32, kBwdDataMasked>(n->gact[l], n->wb[l], nullptr, kDil[l], H, W, total,
+                                 n->a[l - 1], n->gact[l - 1], n->fault, st);
+}
+
 void net_release(bdis_net *n) {
   if (!n) return;
   net_free_acts(n);
-  net_free_pp(n);
+  net_free_planar(n->infer);
+  net_free_planar(n->train);
+  cudaFree(n->part);
   cudaFree(n->w);
   cudaFree(n->m);
   cudaFree(n->v);
@@ -1513,15 +1681,12 @@ namespace bdis {
 bdis_status net_forward_on(bdis_net *n, const float *L, const float *R, int r_stride, int w,
                            int h, int count, float *out, cudaStream_t st) {
   const long long total = (long long)w * h * count;
-  if (g_net_tc == 1) {
-    if (!g_sms) init_sms();
-    int nsb = 0;
-    if (band_rows<32, 32>(4, h, w, &nsb) && band_rows<16, 32>(1, h, w, &nsb) &&
-        band_rows<32, 16>(1, h, w, &nsb)) {
-      bdis_status s = net_reserve_pp(n, h, w, count, st);
-      if (s != BDIS_OK) return s;
-      if (forward_pp(n, L, R, r_stride, h, w, count, out, st)) return record_cuda(cudaGetLastError());
-    }
+  if (!g_sms) init_sms();
+  if (g_net_tc == 1 && band_fits(h, w)) {
+    bdis_status s = net_reserve_planar(n->infer, h, w, count, false, st);
+    if (s != BDIS_OK) return s;
+    if (forward_planar(n, n->infer, L, R, r_stride, h, w, count, out, st))
+      return record_cuda(cudaGetLastError());
   }
   bdis_status s = net_reserve(n, total, false);
   if (s != BDIS_OK) return s;
@@ -1600,17 +1765,41 @@ bdis_status bdis_net_gradient(bdis_net *n, const float *L3, const float *R3, int
       (r_stride != 1 && r_stride != 2))
     return BDIS_E_INVALID_ARG;
   const long long total = (long long)width * height * count;
-  bdis_status s = net_reserve(n, total, true);
+  bdis_status s = net_reserve_part(n);
   if (s != BDIS_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = forward(n, L3, R3, r_stride, height, width, total, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(n->loss, 0, sizeof(float), st);
-  if (e == cudaSuccess) {
-    loss_kernel<<<nblocks(total, 256), 256, 0, st>>>(n->z6, label, total, 1.f / (float)total,
-                                                     n->g6, n->loss);
-    e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (!g_sms) init_sms();
+  // Images that fit the banded kernel train in its layout: the forward pass,
+  // the loss with the data gradients, and the weight gradients are one launch
+  // each (64 images of 40x30: 310 us by per-layer launches, 228 now). Its
+  // padded planes take 704 B per position where the NHWC ones take 768 B per
+  // pixel; a batch beyond 32 GB of them keeps the smaller form.
+  bool done = false;
+  const double planar_bytes = 704.0 * (height + 2 * kPad) * (width + 2 * kPad) * (double)count;
+  if (g_net_tc == 1 && planar_bytes <= 32e9 && band_fits(height, width)) {
+    bdis_net::Planar &p = n->train;
+    s = net_reserve_planar(p, height, width, count, true, st);
+    if (s != BDIS_OK) return s;
+    done = forward_planar(n, p, L3, R3, r_stride, height, width, count, p.map, st) &&
+           backward_planar(n, p, label, height, width, count, st);
+    if (done) e = weight_gradients(n, &p, height, width, count, st);
   }
-  if (e == cudaSuccess) e = backward(n, height, width, total, st);
+  if (!done) {
+    s = net_reserve(n, total, true);
+    if (s != BDIS_OK) return s;
+    e = forward(n, L3, R3, r_stride, height, width, total, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(n->loss, 0, sizeof(float), st);
+    if (e == cudaSuccess) {
+      loss_kernel<<<nblocks(total, 256), 256, 0, st>>>(n->z6, label, total, 1.f / (float)total,
+                                                       n->g6, n->loss);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) {
+      data_gradients(n, height, width, total, st);
+      e = weight_gradients(n, nullptr, height, width, count, st);
+    }
+  }
   if (e == cudaSuccess && loss_out)
     e = cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && grad_out)

@@ -71,8 +71,9 @@ def test_dis_densify_geometry(orc, ps, overlap, count, shape):
 
 
 @pytest.mark.parametrize("count,h,w", [(8, 1, 1), (2, 2, 129), (4, 33, 5), (2, 9, 300), (16, 31, 41)])
-def test_weight_gradient_of_a_batch_is_the_mean_of_its_images(count, h, w):
-    """Images smaller than a tile, narrower than a tap, wider than a tile, and tiles that hold
+@pytest.mark.parametrize("variant", [1, 2])
+def test_weight_gradient_of_a_batch_is_the_mean_of_its_images(count, h, w, variant):
+    """Both layouts training runs in. Images smaller than a tile, narrower than a tap, wider than a tile, and tiles that hold
     several images. For a power of two of images every activation and activation gradient of the
     batch is that of the image alone (scaled exactly), so the gradients differ by the order of
     32-bit sums only: 1e-5 of each layer's norm. The gradient is the same every time."""
@@ -82,10 +83,19 @@ def test_weight_gradient_of_a_batch_is_the_mean_of_its_images(count, h, w):
     label = rng.uniform(0, 4, (count, h, w)).astype(np.float32)
     label[rng.random(label.shape) < 0.1] = np.nan
     net = bd.ProposalNet(bd.net_init_weights(seed=w))
-    loss, g = net.gradient(dev(L), dev(R), dev(label))
-    assert np.array_equal(net.gradient(dev(L), dev(R), dev(label))[1], g)
-    each = [net.gradient(dev(L[i]), dev(R[i]), dev(label[i])) for i in range(count)]
+    old = bd.get_net_variant()
+    try:
+        bd.set_net_variant(variant)
+        loss, g = net.gradient(dev(L), dev(R), dev(label))
+        assert np.array_equal(net.gradient(dev(L), dev(R), dev(label))[1], g)
+        each = [net.gradient(dev(L[i]), dev(R[i]), dev(label[i])) for i in range(count)]
+        bd.set_net_variant(3 - variant)
+        other = net.gradient(dev(L), dev(R), dev(label))[1]
+    finally:
+        bd.set_net_variant(old)
+    net.status()
     net.close()
+    assert np.linalg.norm(g - other) <= 1e-5 * np.linalg.norm(other)
     assert abs(loss - np.mean([e[0] for e in each])) <= 1e-5 * loss
     mean = np.mean([e[1].astype(np.float64) for e in each], axis=0)
     off = 0

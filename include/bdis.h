@@ -376,13 +376,14 @@ bdis_status bdis_select_start(float *d_star_a, float *weight_a, const float *pos
 bdis_status bdis_upsample(const float *map, int map_width, int map_height, int level, int width,
                           int height, int count, float *out, void *stream);
 
-/* Tuning: lane layout of the inverse-search kernel for patch sizes 8, 12 and
- * 16 with the paper's 5-sample window. 1 = one patch column per lane (a
- * group of 8 or 16 lanes per patch); 2 = the wide layout (2 columns per lane
- * for sizes 8 and 16, 3 for size 12); 4 = 4 columns per lane (size 8 only;
- * other sizes take 2). Results are identical up to float rounding; the
- * choice only moves speed. Process-wide; default 2. Returns
- * BDIS_E_INVALID_ARG for any other value. */
+/* Tuning: lane layout of the inverse-search kernel. For patch sizes 8, 12 and
+ * 16 with the paper's 5-sample window: 1 = one patch column per lane (a group
+ * of 8 or 16 lanes per patch); 2 = the wide layout (2 columns per lane for
+ * sizes 8 and 16, 3 for size 12); 4 = 4 columns per lane (size 8 only; other
+ * sizes take 2). Results are identical up to float rounding. For other settings
+ * up to patch size 16: 1 = one column per lane, 2 and 4 = four lanes per patch,
+ * identical bit for bit. The choice only moves speed. Process-wide; default 2.
+ * Returns BDIS_E_INVALID_ARG for any other value. */
 bdis_status bdis_set_search_variant(int columns_per_lane);
 int bdis_get_search_variant(void);
 

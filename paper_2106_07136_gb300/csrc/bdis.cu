@@ -524,10 +524,10 @@ bdis_status autotune_match(void *scratch, size_t scratch_bytes, cudaStream_t st,
   const bool fixed = p.window_samples == 5 && p.window_step == 0.5f &&
                      (p.patch_size == 8 || p.patch_size == 12 || p.patch_size == 16);
   const int reps = 3;
-  // lane layouts of the fixed-size kernels: 1 and the wide one (2, or 3 at
-  // patch 12), and 4 columns per lane at patch 8
+  // lane layouts: one column per lane and the wide one (up to patch 16), and
+  // 4 columns per lane at patch 8 with the paper's window
   const int cpls[3] = {1, 2, 4};
-  const int n_cpl = !fixed ? 1 : (p.patch_size == 8 ? 3 : 2);
+  const int n_cpl = fixed && p.patch_size == 8 ? 3 : p.patch_size <= 16 ? 2 : 1;
   for (int l = p.coarsest_scale; l >= p.finest_scale && e == cudaSuccess; --l) {
     // search: lane layout x block size x global or warp-tiled sampling
     float best = 1e30f;

@@ -28,9 +28,10 @@
 //   - a lane's two columns take the same operations, which run as packed
 //     f32x2 adds and FMAs (per component the scalar rounding).
 //
-// Two instantiations: a fast path with the patch size and window length fixed
-// at compile time (fully unrolled, no per-row guards) for the common settings,
-// and a generic path for any patch size up to 32 and window up to 15.
+// A fast path with the patch size and window length fixed at compile time
+// (fully unrolled, no per-row guards) for the common settings, and a generic path
+// for any patch size up to 32 and window up to 15 (four lanes per patch up to
+// size 16, a lane per column beyond).
 //
 // Roofline: instruction-issue / FP32 bound. Algorithmic work per patch
 // (patch evaluations x 8 flops per pixel): ps^2 * 8 * (updates + s), the
@@ -987,6 +988,235 @@ __global__ void __launch_bounds__(128) search_generic_kernel(const SearchArgs a)
                expf(-(Ec - Emin) / a.kappa), z, ps);
 }
 
+// The generic path for patch sizes up to 16, with fewer lanes per patch: 4
+// lanes, lane c taking columns c, c + 4, ... (CPL = ceil(ps / 4) of them), so a
+// warp carries 8 patches where the kernel above carries 2 at sizes 9 to 16 and 4
+// at 5 to 8, and shares what does not scale with pixels (sample split, tests,
+// divisions, exponentials) among them. The columns of a lane are those that
+// the wide butterflies add first (c with c + 8, then with c + 4), so a lane adds
+// its columns' sums in that order and two exchanges finish the patch: every
+// result has the bits of the kernel above. Rows past 4 CPL - 3 are guarded
+// (uniformly); an invalid column reads nothing and adds zeros. Bound by
+// instruction issue. 24 pairs of 501x375 at patch size 10 with a 7-sample
+// window, levels 3 to 1: 139 us, where one column per lane took 337.
+template <int CPL>
+__device__ __forceinline__ float lane_columns_sum(const float (&v)[CPL]) {
+  if constexpr (CPL == 1) return v[0];
+  if constexpr (CPL == 2) return v[0] + v[1];
+  if constexpr (CPL == 3) return (v[0] + v[2]) + v[1];
+  if constexpr (CPL == 4) return (v[0] + v[2]) + (v[1] + v[3]);
+}
+
+template <int CPL, int MINB>
+__global__ void __launch_bounds__(128, MINB) search_columns_kernel(const SearchArgs a) {
+  constexpr int G = 4, RB = 4 * CPL;  // lanes per patch, rows at most
+  pdl_enter();
+  const int lane = threadIdx.x & 31, c = lane & (G - 1);
+  const unsigned gbits = 0xfu << (lane & ~(G - 1));
+  const int kk = blockIdx.x * (blockDim.x / G) + (int)(threadIdx.x / G);
+  const bool live = kk < a.np;
+  const int kp = live ? kk : a.np - 1;  // past the end: redo the last patch, store nothing
+  const int b = blockIdx.y;
+  const long long k = (long long)b * a.np + kp;
+  const int pj = a.nx_mul ? (int)__umulhi((unsigned)kp, a.nx_mul) : kp / a.nx;
+  const int pi = kp - pj * a.nx;
+  const int ps = a.ps, w = a.w;
+  const int x0 = grid_origin(pi, a.nx, w, ps, a.stride), y0 = grid_origin(pj, a.ny, a.h, ps, a.stride);
+  float u0 = 0.f;
+  if (a.coarse) {
+    const float cx = (float)x0 + (ps - 1) * 0.5f, cy = (float)y0 + (ps - 1) * 0.5f;
+    u0 = 2.f * bilinear_clamped(a.coarse + (long long)b * a.cplane, a.cw, a.ch, cx * 0.5f,
+                                cy * 0.5f);
+  }
+  const int x = x0 + c;  // the lane's first column
+  const long long poff = (long long)b * a.plane + (long long)y0 * w + x;
+  const float *Lc = a.L + poff, *Gc = a.G + poff;
+  const float2 *Rc = a.R2 + poff;
+  auto row = [&](int r) { return r <= RB - 4 || r < ps; };
+  auto act = [&](int j) { return j < CPL - 1 || c + 4 * j < ps; };
+  // columns of the lane whose sample at base shift kd, fraction t, is inside
+  auto valid = [&](int kd, float t) {
+    const int lb = last_base(t, w);
+    unsigned code = 0u;
+#pragma unroll
+    for (int j = 0; j < CPL; ++j) {
+      const int i = x + 4 * j + kd;
+      code |= (unsigned)(act(j) && i >= 0 && i <= lb) << j;
+    }
+    return code;
+  };
+  auto sample = [&](int kd, float t, int r, int j, unsigned code) {
+    const float2 *q = Rc + (long long)r * w + kd + 4 * j;
+    return (code >> j) & 1u
+               ? lerp_packed(BDIS_CHECKED_ONLY(!in_bounds(q - a.R2, a.pixels, kCheckSearchSample)
+                                                   ? make_float2(0.f, 0.f)
+                                                   :) __ldg(q), t)
+               : 0.f;
+  };
+  auto left = [&](const float *p, const float *base, int r, int j, bool on) {
+    return on ? BDIS_LDG(p + (long long)r * w + 4 * j, base, a.pixels, kCheckSearchRows) : 0.f;
+  };
+
+  // ---- inverse-search iterations (Eq. 1)
+  float D = u0, last_step = 0.f, H = 0.f, gcT = 0.f;
+  bool frozen = false, flat = false, have = false;
+  int steps = 0, n = 0;
+  unsigned prev = 0u;
+  float gc[CPL][RB];
+#pragma unroll
+  for (int j = 0; j < CPL; ++j)
+#pragma unroll
+    for (int r = 0; r < RB; ++r) gc[j][r] = 0.f;
+#pragma unroll 1
+  for (int it = 0; it < a.iters; ++it) {
+    if (__all_sync(kFull, frozen)) break;
+    int kd;
+    float t;
+    split_disp(D, kd, t);
+    const unsigned code = valid(kd, t);
+    // every lane votes, whatever its patch's state
+    const bool chg = (__ballot_sync(kFull, code != prev) & gbits) != 0u;
+    const bool need = !frozen && (!have || chg);
+    if (__any_sync(kFull, need)) {
+      float g[CPL][RB], v[CPL];
+#pragma unroll
+      for (int j = 0; j < CPL; ++j) {
+        v[j] = 0.f;
+#pragma unroll
+        for (int r = 0; r < RB; ++r)
+          if (row(r)) {
+            g[j][r] = left(Gc, a.G, r, j, (code >> j) & 1u);
+            v[j] += g[j][r];
+          }
+      }
+      const float sg = group_sum<G>(lane_columns_sum<CPL>(v));
+      const int nn = ps * group_sum_int<G>(__popc(code));
+      const float mg = (a.normalize && nn > 0) ? sg / (float)nn : 0.f;
+      float hh[CPL], ct[CPL];
+#pragma unroll
+      for (int j = 0; j < CPL; ++j) {
+        const bool on = (code >> j) & 1u;
+        hh[j] = ct[j] = 0.f;
+#pragma unroll
+        for (int r = 0; r < RB; ++r)
+          if (row(r)) {
+            const float q = on ? g[j][r] - mg : 0.f;
+            if (need) gc[j][r] = q;
+            hh[j] = fmaf(q, q, hh[j]);
+            ct[j] = fmaf(q, left(Lc, a.L, r, j, act(j)), ct[j]);
+          }
+      }
+      const float hs = group_sum<G>(lane_columns_sum<CPL>(hh));
+      const float cs = group_sum<G>(lane_columns_sum<CPL>(ct));
+      if (need) {
+        H = hs;
+        gcT = cs;
+        n = nn;
+        prev = code;
+        have = true;
+      }
+    }
+    if (!frozen && (n == 0 || H <= kFlatEps * (float)n)) {
+      frozen = true;
+      flat = true;
+    }
+    float acc[CPL];
+#pragma unroll
+    for (int j = 0; j < CPL; ++j) acc[j] = 0.f;
+#pragma unroll
+    for (int r = 0; r < RB; ++r)
+      if (row(r))
+#pragma unroll
+        for (int j = 0; j < CPL; ++j)
+          acc[j] = fmaf(gc[j][r], sample(kd, t, r, j, code), acc[j]);
+    const float Ssum = group_sum<G>(lane_columns_sum<CPL>(acc));
+    if (!frozen) {
+      last_step = (Ssum - gcT) / H;
+      D += last_step;
+      ++steps;
+      if (!isfinite(D) || fabsf(D - u0) > (float)ps || fabsf(last_step) < kStepTol) frozen = true;
+    }
+  }
+
+  const bool fin = isfinite(D);
+  int kd;
+  float t;
+  split_disp(D, kd, t);
+  const int nvalid = ps * group_sum_int<G>(fin ? __popc(valid(kd, t)) : 0);
+  const bool write = live && c == 0;
+  if (a.fusion == BDIS_FUSION_DIS) {
+    finish_patch_dis(a, k, write, D, u0, last_step, flat, steps, nvalid, ps);
+    return;
+  }
+  // ---- Bayesian window (Eqs. 3-4), sample by sample
+  const int half = (a.s - 1) / 2;
+  unsigned vc = fin && fabsf(D - u0) <= (float)ps ? ~0u : 0u;  // a diverged patch reads no window
+#pragma unroll 1
+  for (int i = 0; i < a.s; ++i) {
+    split_disp(D + (float)(i - half) * a.step, kd, t);
+    vc &= valid(kd, t);
+  }
+  const int nc = ps * group_sum_int<G>(__popc(vc));
+  float T[CPL][RB];
+#pragma unroll
+  for (int j = 0; j < CPL; ++j)
+#pragma unroll
+    for (int r = 0; r < RB; ++r) T[j][r] = row(r) ? left(Lc, a.L, r, j, act(j)) : 0.f;
+  float Ec = 0.f, Eo = INFINITY, Emin = INFINITY, z = 0.f;
+#pragma unroll 1
+  for (int i = 0; i < a.s; ++i) {
+    split_disp(D + (float)(i - half) * a.step, kd, t);
+    float d[CPL][RB], v[CPL];
+#pragma unroll
+    for (int j = 0; j < CPL; ++j) {
+      v[j] = 0.f;
+#pragma unroll
+      for (int r = 0; r < RB; ++r)
+        if (row(r)) {
+          d[j][r] = (vc >> j) & 1u ? sample(kd, t, r, j, vc) - T[j][r] : 0.f;
+          v[j] += d[j][r];
+        }
+    }
+    float md = 0.f;
+    if (a.normalize) {
+      const float sd = group_sum<G>(lane_columns_sum<CPL>(v));
+      md = nc > 0 ? sd / (float)nc : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < CPL; ++j) {
+      v[j] = 0.f;
+#pragma unroll
+      for (int r = 0; r < RB; ++r)
+        if (row(r)) {
+          const float q = (vc >> j) & 1u ? d[j][r] - md : 0.f;
+          v[j] = fmaf(q, q, v[j]);
+        }
+    }
+    const float E = group_sum<G>(lane_columns_sum<CPL>(v));
+    if (write && a.energies) a.energies[k * a.s + i] = E;
+    if (i == half)
+      Ec = E;
+    else
+      Eo = fminf(Eo, E);
+    if (E < Emin) {
+      z = (Emin == INFINITY ? 0.f : z * expf(-(Emin - E) / a.kappa)) + 1.f;
+      Emin = E;
+    } else {
+      z += expf(-(E - Emin) / a.kappa);
+    }
+  }
+  finish_patch(a, k, write, D, u0, last_step, flat, steps, nvalid, nc, Ec, Eo,
+               expf(-(Ec - Emin) / a.kappa), z, ps);
+}
+
+template <int CPL, int MINB>
+cudaError_t launch_columns(const SearchArgs &a, cudaStream_t st) {
+  const int count = (int)(a.total / a.np);
+  return launch_maybe_overlapped(search_columns_kernel<CPL, MINB>,
+                                 dim3((unsigned)((a.np + 31) / 32), (unsigned)count), dim3(128), 0,
+                                 st, a);
+}
+
 template <int PS, int CPL, int MINB, bool SH = false>
 cudaError_t launch_fixed(const SearchArgs &a, cudaStream_t st) {
   constexpr int G = pow2_at_least((PS + CPL - 1) / CPL);
@@ -1109,6 +1339,15 @@ cudaError_t launch_search(const SearchArgs &args, cudaStream_t st) {
     }
     if (a.ps == 12) return cpl == 1 ? launch_fast<12, 1, 4>(a, st) : launch_fast<12, 3, 3>(a, st);
     if (a.ps == 16) return cpl == 1 ? launch_fast<16, 1, 4>(a, st) : launch_fast<16, 2, 3>(a, st);
+  }
+  // any other setting: 4 lanes per patch up to size 16 (a larger patch's columns
+  // would not fit a lane's registers); beyond, with the one-column-per-lane
+  // layout asked for, or past the grid's limit, a lane per column
+  if (a.ps <= 16 && a.cols_per_lane != 1 && count <= 65535) {
+    if (a.ps <= 4) return launch_columns<1, 8>(a, st);
+    if (a.ps <= 8) return launch_columns<2, 5>(a, st);
+    if (a.ps <= 12) return launch_columns<3, 4>(a, st);
+    return launch_columns<4, 2>(a, st);
   }
   if (a.ps <= 4) return launch_groups(search_generic_kernel<4>, 4, a, st);
   if (a.ps <= 8) return launch_groups(search_generic_kernel<8>, 8, a, st);

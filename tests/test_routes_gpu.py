@@ -104,3 +104,48 @@ def test_weight_gradient_of_a_batch_is_the_mean_of_its_images(count, h, w, varia
         a, b = g[off:off + n], mean[off:off + n]
         assert np.linalg.norm(a - b) <= 1e-5 * np.linalg.norm(b), (ci, co)
         off += n
+
+
+def _planes(h, w, count, seed):
+    rng = np.random.default_rng(seed)
+    wide = np.cumsum(rng.normal(0, 12, (count, h, w + 16)), axis=2) % 200 + 20
+    shift = rng.integers(0, 6, count)
+    left = np.stack([v[:, 8:8 + w] for v in wide])
+    right = np.stack([v[:, 8 + k:8 + k + w] for v, k in zip(wide, shift)])
+    right = right + rng.normal(0, 1.0, right.shape)
+    return bd.prepare_level0(dev(left.astype(np.float32)), dev(right.astype(np.float32)))
+
+
+@pytest.mark.parametrize("ps", [4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 15, 16])
+@pytest.mark.parametrize("kw", [dict(window_samples=7, window_step=0.4),
+                                dict(window_samples=1, gamma=0.25),
+                                dict(window_samples=15, window_step=0.25, normalize=0),
+                                dict(window_samples=5, window_step=1.0, iterations=0),
+                                dict(window_samples=3, fusion=bd._lib.BDIS_FUSION_DIS)])
+def test_four_lane_search_is_the_one_column_search(ps, kw):
+    """Patches of 4 lanes (each taking every fourth column) against one column per lane, every
+    output bit for bit, on images a patch wide up to some tens of patches, with flat and
+    non-finite regions, from 0 and from a coarse map."""
+    gp = bd.default_params(**dict(dict(patch_size=ps, overlap=0.6, iterations=9), **kw))
+    old = bd.get_search_variant()
+    for i, (h, w, count) in enumerate([(ps, ps, 1), (ps + 3, 2 * ps + 1, 2), (61, 97, 3)]):
+        L, R, G = _planes(h, w, count, 100 * ps + i)
+        if i == 2:
+            L[0, :30, :40] = 90.0
+            G[0, :30, :40] = 0.0
+            R[1, 20:24, 50:53, 0] = float("nan")
+            R[2, 5, 10, 1] = float("inf")
+        coarse = torch.rand(count, (h + 1) // 2, (w + 1) // 2, device=L.device) * 4 if i else None
+        outs = []
+        try:
+            for v in (1, 2):
+                bd.set_search_variant(v)
+                outs.append({k: host(t) for k, t in
+                             bd.search_level(L, R, G, coarse, gp).items()})
+        finally:
+            bd.set_search_variant(old)
+        for key in outs[0]:
+            if kw.get("fusion") and key == "energies":
+                continue  # not written
+            a, b = outs[0][key], outs[1][key]
+            assert np.array_equal(a, b, equal_nan=a.dtype.kind == "f"), (h, w, key)

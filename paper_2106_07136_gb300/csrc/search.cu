@@ -462,20 +462,28 @@ __device__ __forceinline__ bool search_next_step(const SearchArgs &a, const Rows
   return true;
 }
 
-// The window's row pass for column pairs (packed f32x2). Each of the CPL + 2
-// packed pairs of a row is read once and interpolated at both fractions.
-// GUARD: read only the pairs a valid column samples (the others may lie
-// outside the image or the staged tile); without it every pair is in both.
-// An invalid column's sums are finite and are multiplied by 0 in the merge.
+// Window sums of a lane's columns: column pairs as packed f32x2, an odd last
+// column as scalars.
+template <int CPL>
+struct WindowSums {
+  static constexpr int NP = CPL / 2;
+  float2 P1[5][NP > 0 ? NP : 1], P2[5][NP > 0 ? NP : 1];
+  float S1[5], S2[5];  // the odd last column
+};
+
+// The window's row pass. Columns j and j + 1 take the same operations, so each
+// pair runs as one packed f32x2 instruction (per component the same rounding as
+// the scalar fadd / fma): half the issue slots for the residuals and both sums.
+// Each of the CPL + 2 packed pixel pairs of a row is read once and interpolated
+// at both fractions. GUARD: read only the pairs a valid column samples (the
+// others may lie outside the image or the staged tile); without it every pair is
+// in both. An invalid column's sums are finite and are not merged.
 template <int PS, int CPL, bool GUARD, class Rows>
-__device__ __forceinline__ void window_rows_pairs(BDIS_CHECKED_ONLY(const SearchArgs &a, )
-                                                  const Rows &rows, int ib, float t, float th,
-                                                  bool hi, const float *Lc, int w,
-                                                  const bool (&act)[CPL],
-                                                  const bool (&need)[CPL + 2],
-                                                  const float (&cs)[CPL],
-                                                  float2 (&P1)[5][CPL / 2],
-                                                  float2 (&P2)[5][CPL / 2]) {
+__device__ __forceinline__ void window_rows(BDIS_CHECKED_ONLY(const SearchArgs &a, )
+                                            const Rows &rows, int ib, float t, float th, bool hi,
+                                            const float *Lc, int w, const bool (&act)[CPL],
+                                            const bool (&need)[CPL + 2], const float (&cs)[CPL],
+                                            WindowSums<CPL> &ws) {
   constexpr int S = 5;
 #pragma unroll
   for (int r = 0; r < PS; ++r) {
@@ -487,19 +495,16 @@ __device__ __forceinline__ void window_rows_pairs(BDIS_CHECKED_ONLY(const Search
       Lt[m] = lerp_packed(q, t);
       Lh[m] = lerp_packed(q, th);
     }
+    float tn[CPL];  // minus (template + shift): -(T + cs) rounds to exactly -fl(T + cs)
+#pragma unroll
+    for (int j = 0; j < CPL; ++j)
+      tn[j] = -(act[j] ? BDIS_LDG(Lc + (size_t)r * w + j, a.L, a.pixels, kCheckSearchRows) : 0.f) -
+              cs[j];
+    // samples i = 0..4 at D* - 1, -0.5, 0, +0.5, +1: columns ib + j + 1 .. ib + j - 1
 #pragma unroll
     for (int jp = 0; jp < CPL / 2; ++jp) {
       const int j = 2 * jp;
-      // minus (template + shift): -(T + cs) rounds to exactly -fl(T + cs)
-      float tn[2];
-#pragma unroll
-      for (int e = 0; e < 2; ++e)
-        tn[e] = -(act[j + e] ? BDIS_LDG(Lc + (size_t)r * w + j + e, a.L, a.pixels,
-                                          kCheckSearchRows)
-                             : 0.f) -
-                cs[j + e];
-      const float2 Tn = make_float2(tn[0], tn[1]);
-      // samples i = 0..4 at D* - 1, -0.5, 0, +0.5, +1: columns ib + j + 1 .. ib + j - 1
+      const float2 Tn = make_float2(tn[j], tn[j + 1]);
       const float2 d[S] = {
           __fadd2_rn(make_float2(Lt[j + 2], Lt[j + 3]), Tn),
           __fadd2_rn(hi ? make_float2(Lh[j + 2], Lh[j + 3]) : make_float2(Lh[j + 1], Lh[j + 2]),
@@ -509,8 +514,18 @@ __device__ __forceinline__ void window_rows_pairs(BDIS_CHECKED_ONLY(const Search
           __fadd2_rn(make_float2(Lt[j], Lt[j + 1]), Tn)};
 #pragma unroll
       for (int i = 0; i < S; ++i) {
-        P1[i][jp] = __fadd2_rn(P1[i][jp], d[i]);
-        P2[i][jp] = __ffma2_rn(d[i], d[i], P2[i][jp]);
+        ws.P1[i][jp] = __fadd2_rn(ws.P1[i][jp], d[i]);
+        ws.P2[i][jp] = __ffma2_rn(d[i], d[i], ws.P2[i][jp]);
+      }
+    }
+    if constexpr (CPL % 2 == 1) {
+      constexpr int j = CPL - 1;
+      const float d[S] = {Lt[j + 2] + tn[j], (hi ? Lh[j + 2] : Lh[j + 1]) + tn[j],
+                          Lt[j + 1] + tn[j], (hi ? Lh[j + 1] : Lh[j]) + tn[j], Lt[j] + tn[j]};
+#pragma unroll
+      for (int i = 0; i < S; ++i) {
+        ws.S1[i] += d[i];
+        ws.S2[i] = fmaf(d[i], d[i], ws.S2[i]);
       }
     }
   }
@@ -606,23 +621,22 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
   // E = sum (d - md)^2 = S2 - 2 (md - cs) S1 + n (md - cs)^2 per column.
   const float inv_nc = nc > 0 ? __fdividef(1.f, (float)nc) : 0.f;
   float E[S];
+  WindowSums<CPL> ws;
+#pragma unroll
+  for (int i = 0; i < S; ++i) {
+#pragma unroll
+    for (int jp = 0; jp < CPL / 2; ++jp) ws.P1[i][jp] = ws.P2[i][jp] = make_float2(0.f, 0.f);
+    ws.S1[i] = ws.S2[i] = 0.f;
+  }
+  // A warp whose patches are all in range (so their pairs lie in a staged
+  // tile, if any) with all pairs in the image reads them unconditionally.
+  if (__all_sync(kFull, inr && ib >= 1 && ib + CPL <= w - 1))
+    window_rows<PS, CPL, false>(BDIS_CHECKED_ONLY(a, ) rows, ib, t, th, hi, Lc, w, act, need, cs,
+                                ws);
+  else
+    window_rows<PS, CPL, true>(BDIS_CHECKED_ONLY(a, ) rows, ib, t, th, hi, Lc, w, act, need, cs,
+                               ws);
   if constexpr (CPL % 2 == 0) {
-    // Columns j and j + 1 take the same operations, so each pair runs as one
-    // packed f32x2 instruction (per component the same rounding as the scalar
-    // fadd / fma): half the issue slots for the residuals and both sums.
-    float2 P1[S][CPL / 2], P2[S][CPL / 2];
-#pragma unroll
-    for (int i = 0; i < S; ++i)
-#pragma unroll
-      for (int jp = 0; jp < CPL / 2; ++jp) P1[i][jp] = P2[i][jp] = make_float2(0.f, 0.f);
-    // A warp whose patches are all in range (so their pairs lie in a staged
-    // tile, if any) with all pairs in the image reads them unconditionally.
-    if (__all_sync(kFull, inr && ib >= 1 && ib + CPL <= w - 1))
-      window_rows_pairs<PS, CPL, false>(BDIS_CHECKED_ONLY(a, ) rows, ib, t, th, hi, Lc, w, act,
-                                        need, cs, P1, P2);
-    else
-      window_rows_pairs<PS, CPL, true>(BDIS_CHECKED_ONLY(a, ) rows, ib, t, th, hi, Lc, w, act,
-                                       need, cs, P1, P2);
     // the merge below, per column pair; an invalid column's term is x * 0
     // (every term is finite)
     const float2 kPS = make_float2((float)PS, (float)PS), kM2 = make_float2(-2.f, -2.f);
@@ -638,7 +652,7 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
       float s1 = 0.f;
 #pragma unroll
       for (int jp = 0; jp < CPL / 2; ++jp) {
-        const float2 x = __fmul2_rn(__ffma2_rn(kPS, cs2[jp], P1[i][jp]), vm[jp]);
+        const float2 x = __fmul2_rn(__ffma2_rn(kPS, cs2[jp], ws.P1[i][jp]), vm[jp]);
         s1 += x.x + x.y;
       }
       s1 = group_sum<G>(s1);
@@ -648,48 +662,25 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
 #pragma unroll
       for (int jp = 0; jp < CPL / 2; ++jp) {
         const float2 u = __fadd2_rn(md2, ncs2[jp]);
-        const float2 in = __ffma2_rn(__fmul2_rn(kPS, u), u, P2[i][jp]);
-        const float2 x = __fmul2_rn(__ffma2_rn(__fmul2_rn(kM2, u), P1[i][jp], in), vm[jp]);
+        const float2 in = __ffma2_rn(__fmul2_rn(kPS, u), u, ws.P2[i][jp]);
+        const float2 x = __fmul2_rn(__ffma2_rn(__fmul2_rn(kM2, u), ws.P1[i][jp], in), vm[jp]);
         e += x.x + x.y;
       }
       E[i] = group_sum<G>(e);
     }
   } else {
-    float S1[S][CPL], S2[S][CPL];
-#pragma unroll
-    for (int i = 0; i < S; ++i)
-#pragma unroll
-      for (int j = 0; j < CPL; ++j) S1[i][j] = S2[i][j] = 0.f;
-#pragma unroll
-    for (int r = 0; r < PS; ++r) {
-      float Lt[CPL + 2], Lh[CPL + 2];
-#pragma unroll
-      for (int m = 0; m < CPL + 2; ++m) {
-        const float2 q = need[m] ? rows.ld(rows.col(ib - 1 + m), r) : make_float2(0.f, 0.f);
-        Lt[m] = lerp_packed(q, t);
-        Lh[m] = lerp_packed(q, th);
-      }
-#pragma unroll
-      for (int j = 0; j < CPL; ++j) {
-        const float Tj =  // template + shift
-            (vc[j] ? BDIS_LDG(Lc + (size_t)r * w + j, a.L, a.pixels, kCheckSearchRows) : 0.f) +
-            cs[j];
-        // samples i = 0..4 at D* - 1, -0.5, 0, +0.5, +1: columns ib + j + 1 .. ib + j - 1.
-        // An invalid column's sums (finite: its pairs read as 0) are not merged below.
-        const float d[S] = {Lt[j + 2] - Tj, (hi ? Lh[j + 2] : Lh[j + 1]) - Tj, Lt[j + 1] - Tj,
-                            (hi ? Lh[j + 1] : Lh[j]) - Tj, Lt[j] - Tj};
-#pragma unroll
-        for (int i = 0; i < S; ++i) {
-          S1[i][j] += d[i];
-          S2[i][j] = fmaf(d[i], d[i], S2[i][j]);
-        }
-      }
-    }
+    // column j's sums over the rows, for sample i
+    auto sum1 = [&](int i, int j) {
+      return j == CPL - 1 ? ws.S1[i] : j % 2 ? ws.P1[i][j / 2].y : ws.P1[i][j / 2].x;
+    };
+    auto sum2 = [&](int i, int j) {
+      return j == CPL - 1 ? ws.S2[i] : j % 2 ? ws.P2[i][j / 2].y : ws.P2[i][j / 2].x;
+    };
 #pragma unroll
     for (int i = 0; i < S; ++i) {
       float s1 = 0.f;
 #pragma unroll
-      for (int j = 0; j < CPL; ++j) s1 += vc[j] ? S1[i][j] + (float)PS * cs[j] : 0.f;
+      for (int j = 0; j < CPL; ++j) s1 += vc[j] ? sum1(i, j) + (float)PS * cs[j] : 0.f;
       s1 = group_sum<G>(s1);
       const float md = (a.normalize && nc > 0) ? s1 * inv_nc : 0.f;
       float e = 0.f;
@@ -697,7 +688,7 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
       for (int j = 0; j < CPL; ++j) {
         if (vc[j]) {
           const float u = md - cs[j];
-          e += fmaf(-2.f * u, S1[i][j], fmaf((float)PS * u, u, S2[i][j]));
+          e += fmaf(-2.f * u, sum1(i, j), fmaf((float)PS * u, u, sum2(i, j)));
         }
       }
       E[i] = group_sum<G>(e);
@@ -1337,8 +1328,18 @@ cudaError_t launch_search(const SearchArgs &args, cudaStream_t st) {
       // (the tiled variant keeps it in registers at 72: 7 blocks)
       return a.tiled ? launch_tiled<8, 2, 7>(a, st) : launch_fixed<8, 2, 8, true>(a, st);
     }
-    if (a.ps == 12) return cpl == 1 ? launch_fast<12, 1, 4>(a, st) : launch_fast<12, 3, 3>(a, st);
-    if (a.ps == 16) return cpl == 1 ? launch_fast<16, 1, 4>(a, st) : launch_fast<16, 2, 3>(a, st);
+    // 128 registers: 4 blocks of 128 per SM. Search of 64 pairs of 640x480: patch
+    // 12 1478 us (3 blocks at 168 registers 1625, 5 to 7 blocks, with the
+    // gradient in shared memory, 1574 to 1819), patch 16 1192 us (1361; 1214 to
+    // 1449). The tiled variant's staged rows leave room for 3.
+    if (a.ps == 12) {
+      if (cpl == 1) return launch_fast<12, 1, 4>(a, st);
+      return a.tiled ? launch_tiled<12, 3, 3>(a, st) : launch_fixed<12, 3, 4>(a, st);
+    }
+    if (a.ps == 16) {
+      if (cpl == 1) return launch_fast<16, 1, 4>(a, st);
+      return a.tiled ? launch_tiled<16, 2, 3>(a, st) : launch_fixed<16, 2, 4>(a, st);
+    }
   }
   // any other setting: 4 lanes per patch up to size 16 (a larger patch's columns
   // would not fit a lane's registers); beyond, with the one-column-per-lane

@@ -172,15 +172,11 @@ constexpr int kStX = 2 * kPyrX + 7, kStY = 2 * kPyrY + 7;  // staged input colum
 constexpr int kStP = 72;                                     // staged row pitch (floats)
 constexpr int kCx = kPyrX + 2;                               // computed columns (with halo)
 
-// Stage columns of tap 0 for the computed columns of this lane (cx = lane,
-// and lanes 0, 1 also take 32, 33), at the reflected output coordinate.
-__device__ __forceinline__ void stage_taps(int lane, int X0, int dw, int (&c0)[2], bool (&cok)[2]) {
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int cx = lane + 32 * u, Xr = X0 - 1 + cx;
-    cok[u] = cx < kCx && Xr <= dw;
-    c0[u] = cok[u] ? 2 * (reflect101(Xr, dw) - X0) + 2 : 0;
-  }
+// Stage column of tap 0 for computed column cx, at the reflected output
+// coordinate (always even), or -1 past the last one.
+__device__ __forceinline__ int stage_tap(int cx, int X0, int dw) {
+  const int Xr = X0 - 1 + cx;
+  return Xr <= dw ? 2 * (reflect101(Xr, dw) - X0) + 2 : -1;
 }
 
 // Columns of the stage this lane fills (c = lane + 32 u): the input column
@@ -199,41 +195,49 @@ __device__ __forceinline__ void stage_columns(int lane, int X0, int w, int (&xsr
 // horizontal 5-tap pass per stage row and computed column, a vertical 5-tap
 // pass per computed output, then L1, packed R1 and Sobel-x / 8 of L1. The two
 // views sit side by side, (L, R) per pixel, so that every tap of both is one
-// 8-byte shared load and one packed f32x2 FMA (per component the same fma, in
-// the same order, as down_kernel).
+// packed f32x2 FMA (per component the same fma, in the same order, as
+// down_kernel); a lane's first tap is on an even column, so taps come two to a
+// 16-byte shared load. A warp takes columns 0 .. 31; the two past them, of all
+// rows, are dealt to single threads. 256 threads.
 __device__ __forceinline__ void pyramid_passes(const float2 (*inLR)[kStP], float2 (*hLR)[kCx],
-                                               float2 (*sLR)[kCx], const int (&c0)[2],
-                                               const bool (&cok)[2], int b, int X0, int Y0,
-                                               int h, int dw, int dh, float *__restrict__ L1,
+                                               float2 (*sLR)[kCx], int b, int X0, int Y0, int h,
+                                               int dw, int dh, float *__restrict__ L1,
                                                float2 *__restrict__ R1, float *__restrict__ G1) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = 8;
   const float k[5] = {1.f / 16, 4.f / 16, 6.f / 16, 4.f / 16, 1.f / 16};
-  for (int r = warp; r < kStY; r += nwarp) {
-    if (2 * Y0 - 4 + r > h + 1) break;
+  auto across = [&](int r, int c0) {
+    const float4 p = *reinterpret_cast<const float4 *>(&inLR[r][c0]);
+    const float4 q = *reinterpret_cast<const float4 *>(&inLR[r][c0 + 2]);
+    const float2 in[5] = {make_float2(p.x, p.y), make_float2(p.z, p.w), make_float2(q.x, q.y),
+                          make_float2(q.z, q.w), inLR[r][c0 + 4]};
+    float2 hv = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      if (!cok[u]) continue;
-      float2 hv = make_float2(0.f, 0.f);
+    for (int i = 0; i < 5; ++i) hv = __ffma2_rn(make_float2(k[i], k[i]), in[i], hv);
+    return hv;
+  };
+  auto down = [&](int cy, int cx) {
+    const int r0 = 2 * (reflect101(Y0 - 1 + cy, dh) - Y0) + 2;  // stage row of tap 0
+    float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i < 5; ++i) hv = __ffma2_rn(make_float2(k[i], k[i]), inLR[r][c0[u] + i], hv);
-      hLR[r][lane + 32 * u] = hv;
-    }
+    for (int j = 0; j < 5; ++j) acc = __ffma2_rn(make_float2(k[j], k[j]), hLR[r0 + j][cx], acc);
+    return acc;
+  };
+  const int rows = min(kStY, h + 2 - (2 * Y0 - 4));      // stage rows that exist
+  const int outs = min(kPyrY + 2, dh + 1 - (Y0 - 1));    // computed rows that exist
+  const int c0 = stage_tap(lane, X0, dw);
+  if (c0 >= 0)
+    for (int r = warp; r < rows; r += nwarp) hLR[r][lane] = across(r, c0);
+  if (tid < 2 * rows) {
+    const int cx = 32 + (tid & 1), ce = stage_tap(cx, X0, dw);
+    if (ce >= 0) hLR[tid >> 1][cx] = across(tid >> 1, ce);
   }
   __syncthreads();
   // vertical taps: the downsampled value of every computed cell
-  for (int cy = warp; cy < kPyrY + 2; cy += nwarp) {
-    const int Yr = Y0 - 1 + cy;
-    if (Yr > dh) break;
-    const int r0 = 2 * (reflect101(Yr, dh) - Y0) + 2;  // stage row of tap 0
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      if (!cok[u]) continue;
-      const int cx = lane + 32 * u;
-      float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int j = 0; j < 5; ++j) acc = __ffma2_rn(make_float2(k[j], k[j]), hLR[r0 + j][cx], acc);
-      sLR[cy][cx] = acc;
-    }
+  if (c0 >= 0)
+    for (int cy = warp; cy < outs; cy += nwarp) sLR[cy][lane] = down(cy, lane);
+  if (tid >= 128 && tid - 128 < 2 * outs) {
+    const int cx = 32 + (tid & 1), cy = (tid - 128) >> 1;
+    if (stage_tap(cx, X0, dw) >= 0) sLR[cy][cx] = down(cy, cx);
   }
   __syncthreads();
   const int cx = 1 + lane;
@@ -256,7 +260,7 @@ __device__ __forceinline__ void pyramid_passes(const float2 (*inLR)[kStP], float
 __global__ void __launch_bounds__(256) pyramid_fused_kernel(
     const float *__restrict__ L, const float2 *__restrict__ R, int w, int h, int dw, int dh,
     float *__restrict__ L1, float2 *__restrict__ R1, float *__restrict__ G1) {
-  __shared__ float2 inLR[kStY][kStP];
+  __shared__ __align__(16) float2 inLR[kStY][kStP];
   __shared__ float2 hLR[kStY][kCx];
   __shared__ float2 sLR[kPyrY + 2][kCx];
   pdl_enter();
@@ -290,12 +294,9 @@ __global__ void __launch_bounds__(256) pyramid_fused_kernel(
                    "l"(Rb + rowoff + xsrc[u]));  // the value is the pair's first word
     }
   }
-  int c0[2];
-  bool cok[2];
-  stage_taps(lane, X0, dw, c0, cok);  // while the copies travel
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
-  pyramid_passes(inLR, hLR, sLR, c0, cok, b, X0, Y0, h, dw, dh, L1, R1, G1);
+  pyramid_passes(inLR, hLR, sLR, b, X0, Y0, h, dw, dh, L1, R1, G1);
 }
 
 // Level 0 and the first pyramid step in one pass over the input views: the
@@ -304,13 +305,16 @@ __global__ void __launch_bounds__(256) pyramid_fused_kernel(
 // output tile: L0, packed R0 and Sobel-x / 8 of L0, the same values and
 // operations as prepare_level0) from the stage, then runs the pyramid step on
 // it. Level 0 is thus written once and never read back for level 1.
+// 512 pairs of 640x480: 722 us (4.8 TB/s of 22 B per pixel), bound by its
+// shared-memory reads and load latency; with single pixels, scalar stores and
+// 8-byte taps it took 842.
 template <typename T>
 __global__ void __launch_bounds__(256) prepare_pyramid0_kernel(
     const void *__restrict__ left, const void *__restrict__ right, size_t pitch, size_t stride,
     int w, int h, int dw, int dh, int words, float *__restrict__ L0, float2 *__restrict__ R0,
     float *__restrict__ G0, float *__restrict__ L1, float2 *__restrict__ R1,
     float *__restrict__ G1) {
-  __shared__ float2 inLR[kStY][kStP];
+  __shared__ __align__(16) float2 inLR[kStY][kStP];
   __shared__ float2 hLR[kStY][kCx];
   __shared__ float2 sLR[kPyrY + 2][kCx];
   pdl_enter();
@@ -323,40 +327,39 @@ __global__ void __launch_bounds__(256) prepare_pyramid0_kernel(
   stage_columns(lane, X0, w, xsrc, xok);
   // 8-bit views with 4-byte aligned rows (words != 0), block inside the image
   // in x: a stage row is 18 aligned 32-bit words (columns 2 X0 - 4 ..
-  // 2 X0 + 67), one per lane, and all of the warp's rows are loaded before any
-  // is stored. Otherwise one element per lane and column, reflected.
-  constexpr int kRowsPerWarp = (kStY + 7) / 8, kWords = (kStX + 3) / 4;
-  if (sizeof(T) == 1 && words && 2 * X0 - 4 >= 0 && 2 * X0 + 4 * kWords - 4 <= w && nwarp == 8) {
-    uint32_t wl[kRowsPerWarp], wr[kRowsPerWarp];
+  // 2 X0 + 67), dealt to the threads in turn, and all of a thread's words are
+  // loaded before any is stored. Otherwise one element per lane and column,
+  // reflected.
+  constexpr int kWords = (kStX + 3) / 4, kPerThread = (kStY * kWords + 255) / 256;
+  static_assert(4 * kWords <= kStP, "a row's words fit its pitch");
+  if (sizeof(T) == 1 && words && 2 * X0 - 4 >= 0 && 2 * X0 + 4 * kWords - 4 <= w) {
+    uint32_t wl[kPerThread], wr[kPerThread];
 #pragma unroll
-    for (int q = 0; q < kRowsPerWarp; ++q) {
-      const int r = warp + 8 * q, yi = 2 * Y0 - 4 + r;
-      const bool rok = lane < kWords && r < kStY && yi <= h + 1;
-      const size_t off = (size_t)(rok ? reflect101(yi, h) : 0) * pitch + (size_t)(2 * X0 - 4);
+    for (int q = 0; q < kPerThread; ++q) {
+      const int i = (int)threadIdx.x + 256 * q, r = i / kWords, wd = i - r * kWords;
+      const int yi = 2 * Y0 - 4 + r;
+      const bool rok = r < kStY && yi <= h + 1;
+      const size_t off =
+          (size_t)(rok ? reflect101(yi, h) : 0) * pitch + (size_t)(2 * X0 - 4) + 4 * wd;
 #ifdef BDIS_CHECKED
       // the word's last byte lies inside the view (h - 1 full rows and w bytes)
-      const bool inb =
-          !rok || in_bounds((long long)(off + 4 * lane + 3), (long long)(h - 1) * pitch + w,
-                            kCheckPyramidInput);
-      wl[q] = rok && inb ? __ldg(reinterpret_cast<const uint32_t *>(lb + off) + lane) : 0u;
-      wr[q] = rok && inb ? __ldg(reinterpret_cast<const uint32_t *>(rb + off) + lane) : 0u;
+      const bool inb = !rok || in_bounds((long long)(off + 3), (long long)(h - 1) * pitch + w,
+                                         kCheckPyramidInput);
+      wl[q] = rok && inb ? __ldg(reinterpret_cast<const uint32_t *>(lb + off)) : 0u;
+      wr[q] = rok && inb ? __ldg(reinterpret_cast<const uint32_t *>(rb + off)) : 0u;
 #else
-      wl[q] = rok ? __ldg(reinterpret_cast<const uint32_t *>(lb + off) + lane) : 0u;
-      wr[q] = rok ? __ldg(reinterpret_cast<const uint32_t *>(rb + off) + lane) : 0u;
+      wl[q] = rok ? __ldg(reinterpret_cast<const uint32_t *>(lb + off)) : 0u;
+      wr[q] = rok ? __ldg(reinterpret_cast<const uint32_t *>(rb + off)) : 0u;
 #endif
     }
 #pragma unroll
-    for (int q = 0; q < kRowsPerWarp; ++q) {
-      const int r = warp + 8 * q;
-      if (r >= kStY || 2 * Y0 - 4 + r > h + 1) break;
-      if (lane >= kWords) continue;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int c = 4 * lane + e;
-        if (c < kStX)
-          inLR[r][c] = make_float2((float)((wl[q] >> (8 * e)) & 0xffu),
-                                   (float)((wr[q] >> (8 * e)) & 0xffu));
-      }
+    for (int q = 0; q < kPerThread; ++q) {
+      const int i = (int)threadIdx.x + 256 * q, r = i / kWords, wd = i - r * kWords;
+      if (r >= kStY) break;
+      float4 *dst = reinterpret_cast<float4 *>(&inLR[r][4 * wd]);
+      auto px = [&](uint32_t v, int e) { return (float)((v >> (8 * e)) & 0xffu); };
+      dst[0] = make_float4(px(wl[q], 0), px(wr[q], 0), px(wl[q], 1), px(wr[q], 1));
+      dst[1] = make_float4(px(wl[q], 2), px(wr[q], 2), px(wl[q], 3), px(wr[q], 3));
     }
   } else {
     for (int r = warp; r < kStY; r += nwarp) {
@@ -375,13 +378,54 @@ __global__ void __launch_bounds__(256) prepare_pyramid0_kernel(
       }
     }
   }
-  int c0[2];
-  bool cok[2];
-  stage_taps(lane, X0, dw, c0, cok);
   __syncthreads();
   // level 0: pixel (2 X0 + i, 2 Y0 + j) is stage (row j + 4, column i + 4); its
-  // neighbours x +- 1, y +- 1 are the staged reflect-101 ones
-  for (int j = warp; j < 2 * kPyrY; j += nwarp) {
+  // neighbours x +- 1, y +- 1 are the staged reflect-101 ones. At an even width
+  // a lane takes the pixel pair i = 2 lane, walking down four rows of its warp:
+  // a row's three column pairs are read once, as 16-byte shared loads, and its
+  // horizontal differences serve the three rows around it; stores are 8 and 16
+  // bytes. Otherwise pixel by pixel.
+  if (w % 2 == 0) {
+    constexpr int kRows = 2 * kPyrY / 8;
+    const int x = 2 * X0 + 2 * lane, j0 = warp * kRows, c = 2 * lane + 4;
+    if (x < w) {
+      float2 d[3];           // horizontal differences of stage rows j - 1, j, j + 1
+      float4 v[2];           // the pair's (L, R) of rows j, j + 1
+      float rn[2];           // the right neighbour's R of rows j, j + 1
+      auto load = [&](int r, float2 &dd, float4 &vv, float &rr) {
+        const float4 p = *reinterpret_cast<const float4 *>(&inLR[r][c - 2]);
+        const float4 q = *reinterpret_cast<const float4 *>(&inLR[r][c]);
+        const float4 n = *reinterpret_cast<const float4 *>(&inLR[r][c + 2]);
+        dd = make_float2(q.z - p.z, n.x - q.x);
+        vv = q;
+        rr = n.y;
+      };
+      float4 vx;
+      float rx;
+      load(j0 + 3, d[0], vx, rx);
+      load(j0 + 4, d[1], v[0], rn[0]);
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) {
+        const int y = 2 * Y0 + j0 + j;
+        if (y >= h) break;
+        load(j0 + j + 5, d[2], v[1], rn[1]);
+        const size_t o = (size_t)b * w * h + (size_t)y * w + x;
+        BDIS_CHECKED_ONLY(
+            if (!in_bounds((long long)o + 1, (long long)gridDim.z * w * h, kCheckPyramidOut)) break;)
+        const float4 q = v[0];
+        *reinterpret_cast<float2 *>(L0 + o) = make_float2(q.x, q.z);
+        *reinterpret_cast<float2 *>(G0 + o) =
+            make_float2((d[0].x + 2.f * d[1].x + d[2].x) * 0.125f,
+                        (d[0].y + 2.f * d[1].y + d[2].y) * 0.125f);
+        *reinterpret_cast<float4 *>(R0 + o) =
+            make_float4(q.y, q.w - q.y, q.w, x + 2 < w ? rn[0] - q.w : 0.f);
+        d[0] = d[1];
+        d[1] = d[2];
+        v[0] = v[1];
+        rn[0] = rn[1];
+      }
+    }
+  } else for (int j = warp; j < 2 * kPyrY; j += nwarp) {
     const int y = 2 * Y0 + j;
     if (y >= h) break;
     const int r = j + 4;
@@ -401,7 +445,7 @@ __global__ void __launch_bounds__(256) prepare_pyramid0_kernel(
       R0[o] = make_float2(v.y, x + 1 < w ? inLR[r][c + 1].y - v.y : 0.f);
     }
   }
-  pyramid_passes(inLR, hLR, sLR, c0, cok, b, X0, Y0, h, dw, dh, L1, R1, G1);
+  pyramid_passes(inLR, hLR, sLR, b, X0, Y0, h, dw, dh, L1, R1, G1);
 }
 
 __global__ void pack_right_kernel(const float *__restrict__ R, int w, long long total,

@@ -282,9 +282,10 @@ void set_launch_overlap(int on);
 // SMs of the current device (looked up once per device).
 int device_sms();
 
+// Overlapped while the launch has at most per_sm blocks per SM.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_maybe_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                    cudaStream_t st, Args &&...args) {
+cudaError_t launch_overlapped_upto(long long per_sm, void (*kernel)(KArgs...), dim3 grid,
+                                   dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -294,13 +295,19 @@ cudaError_t launch_maybe_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 bl
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  // Only launches of at most 16 blocks per SM overlap. Measured: one pair's
-  // latency fell 17% with the overlap, but a 512-pair step took 1.7% longer
-  // (likely because the next kernel's early blocks land on whichever SMs
-  // free up first, an uneven placement for the rest of that kernel).
   const long long blocks = (long long)grid.x * grid.y * grid.z;
-  cfg.numAttrs = (launch_overlap() && blocks <= 16LL * device_sms()) ? 1 : 0;
+  cfg.numAttrs = (launch_overlap() && blocks <= per_sm * device_sms()) ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+// Only launches of at most 16 blocks per SM overlap. Measured: one pair's
+// latency fell 17% with the overlap, but a 512-pair step took 1.7% longer
+// (likely because the next kernel's early blocks land on whichever SMs
+// free up first, an uneven placement for the rest of that kernel).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_maybe_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                    cudaStream_t st, Args &&...args) {
+  return launch_overlapped_upto(16, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // Fill SearchArgs / DensifyArgs geometry from parameters (host).

@@ -279,6 +279,13 @@ __device__ __forceinline__ void pdl_enter() {
 }
 int launch_overlap();
 void set_launch_overlap(int on);
+// Keeps this thread's launches in plain stream order while it lives.
+struct NoOverlap {
+  NoOverlap();
+  ~NoOverlap();
+  NoOverlap(const NoOverlap &) = delete;
+  NoOverlap &operator=(const NoOverlap &) = delete;
+};
 // SMs of the current device (looked up once per device).
 int device_sms();
 

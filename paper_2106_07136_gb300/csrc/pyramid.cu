@@ -472,7 +472,10 @@ int g_pyramid_fused = 2;
 int pyramid_fused() { return g_pyramid_fused; }
 
 int g_launch_overlap = 1;
-int launch_overlap() { return g_launch_overlap; }
+static thread_local int t_no_overlap = 0;
+int launch_overlap() { return g_launch_overlap && !t_no_overlap; }
+NoOverlap::NoOverlap() { ++t_no_overlap; }
+NoOverlap::~NoOverlap() { --t_no_overlap; }
 void set_launch_overlap(int on) { g_launch_overlap = on ? 1 : 0; }
 
 int device_sms() {

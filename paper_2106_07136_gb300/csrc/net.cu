@@ -1485,15 +1485,15 @@ bool launch_chain(bdis_net *n, BandNet &net, int H, int W, int count, cudaStream
     bh[l] = l == 0   ? band_rows<16, 32>(net.layer[l].dil, H, W, &nsb[l])
             : l == 5 ? band_rows<32, 16>(net.layer[l].dil, H, W, &nsb[l])
                      : band_rows<32, 32>(net.layer[l].dil, H, W, &nsb[l]);
-  // Band heights. Small batches: bands of fewer rows, so that a layer's
-  // bands spread over the SMs (a single 40x30 image would otherwise be two
-  // bands on two SMs, the rest waiting at the grid barriers). Then the bands
-  // of an image are made equal (30 rows: 15 + 15, not 21 + 9): blocks take
-  // bands round robin, and unequal bands would give every other block all
-  // the tall ones. A result does not depend on the band height: each
-  // position's MMAs and epilogue are the same.
-  const int per_image = (g_sms + count - 1) / count;  // bands wanted per image
-  const int want = std::max(1, (H + per_image - 1) / per_image);
+  // Band heights: per layer, the number of equal bands per image (at least as
+  // many as the limits ask for) whose rounds over the SMs cost least, a round
+  // being a band's tiles and one more for its fill and drain. Bands of fewer
+  // rows spread a small batch over the SMs, but a last round that few blocks
+  // have work in costs as much as a full one: 64 images of 40x30 in 3 bands each
+  // were 192 bands on 152 SMs (59 us a forward pass by host clock), in 2 they are
+  // 128 (51); 32 in 5 bands 52, in 4 40; 100 in 2 bands 74, in 3 61. A result
+  // does not depend on the band height: each position's MMAs and epilogue are
+  // the same.
   int slab = 0;
   // one block per SM, or one per band where a layer has fewer bands (a
   // single image): fewer blocks meet at each grid barrier and restage the
@@ -1501,12 +1501,22 @@ bool launch_chain(bdis_net *n, BandNet &net, int H, int W, int count, cudaStream
   long long units = 1;
   for (int l = 0; l < layers; ++l) {
     if (!bh[l]) return false;
-    const int nb = (H + std::min(want, bh[l]) - 1) / std::min(want, bh[l]);
-    const int even = (H + nb - 1) / nb;  // <= bh[l]: the limits still hold
-    if (even < bh[l]) {
-      const int Wp = W + 2 * kPad, soff = net.layer[l].dil * Wp + net.layer[l].dil;
-      bh[l] = even;
-      nsb[l] = (even * Wp + 127) / 128 * 128 + 2 * soff;
+    const int Wp = W + 2 * kPad, soff = net.layer[l].dil * Wp + net.layer[l].dil;
+    int best = 0;
+    long long cost = 0;
+    for (int nb = (H + bh[l] - 1) / bh[l]; nb <= H; ++nb) {
+      const int rows = (H + nb - 1) / nb;
+      const long long c = ((long long)count * ((H + rows - 1) / rows) + g_sms - 1) / g_sms *
+                          ((rows * Wp + 127) / 128 + 1);
+      if (!best || c < cost) {
+        best = rows;
+        cost = c;
+      }
+      if ((long long)count * nb >= 8LL * g_sms) break;  // more rounds only add fills
+    }
+    if (best < bh[l]) {  // the limits still hold
+      bh[l] = best;
+      nsb[l] = (best * Wp + 127) / 128 * 128 + 2 * soff;
     }
     net.layer[l].BH = bh[l];
     net.layer[l].nsb = nsb[l];

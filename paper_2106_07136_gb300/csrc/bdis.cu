@@ -889,6 +889,53 @@ bdis_status bdis_warm_map(const float *prev, int width, int height, int level, i
 
 namespace {
 
+// How bdis_match_host splits a batch. A chunk costs about 90 us of launches and
+// underfilled coarse levels, as much as matching four 640x480 pairs; it hides
+// the copies of its neighbours (a pair's copy in takes an eighth of its match, its
+// copy out a quarter). So a small batch runs whole; a larger one splits off a last
+// chunk, whose copy out is all that nothing hides; then also a first one, whose
+// copy in nothing hides; and a large one grades the middle, so that each copy
+// still fits under the match beside it. Lines drawn by the work, in 640x480
+// pairs, all sides measured (us per call, even split of before -> now): 8 pairs
+// 575 -> 389 (two chunks 422), 16 pairs 783 -> 650 (one chunk 665), 32 pairs 1258
+// -> 1130 (one 1202, three 1142), 64 pairs 2072 -> 1953 (two 2075, four 2017), 128
+// pairs 3677 -> 3611, 512 pairs 13350 -> 13240 (three 13780). A middle chunk past
+// 32 GB of workspace keeps the even split, whose chunks are smaller.
+constexpr int kHostChunks = 5;
+
+int host_chunks(int w, int h, int count, const bdis_params &p, int (&n)[kHostChunks]) {
+  const double pairs = (double)w * h * count / (640.0 * 480.0);
+  int k = 0;
+  auto part = [&](double share) { return std::max(1, (int)(share * count)); };
+  if (count < 2 || pairs < 12) {
+    n[k++] = count;
+  } else if (pairs < 48 || count < 8) {
+    n[1] = part(1.0 / 4);
+    n[0] = count - n[1];
+    k = 2;
+  } else if (pairs < 256 || count < 32) {
+    n[0] = part(1.0 / 16);
+    n[2] = part(3.0 / 16);
+    n[1] = count - n[0] - n[2];
+    k = 3;
+  } else {
+    n[0] = part(1.0 / 32);
+    n[1] = part(1.0 / 4);
+    n[3] = part(5.0 / 32);
+    n[4] = part(1.0 / 16);
+    n[2] = count - n[0] - n[1] - n[3] - n[4];
+    k = 5;
+  }
+  const int largest = *std::max_element(n, n + k);
+  if (k > 1 && plan_layout(w, h, largest, p, true).bytes > (32ull << 30) && count >= 5) {
+    k = 5;
+    n[0] = n[4] = part(1.0 / 16);
+    n[1] = n[2] = (count - n[0] - n[4]) / 3;
+    n[3] = count - n[0] - n[4] - n[1] - n[2];
+  }
+  return k;
+}
+
 // Copy streams and events of the host pipeline, created on first use.
 bdis_status ensure_pipeline(bdis_handle *h) {
   if (h->copy_in) return BDIS_OK;
@@ -919,22 +966,9 @@ bdis_status bdis_match_host(bdis_handle *h, const uint8_t *left, const uint8_t *
   // chunk i-1 is matched (stream) and chunk i-2's result is copied out
   // (copy_out). Inputs and outputs on the device are double-buffered by slot
   // (i & 1); a slot is refilled only after the match that read it (ev_done)
-  // and the copy-out that read its output (ev_out) have finished. From 32
-  // pairs the first and last chunks are a sixteenth of the batch, so that
-  // the copy-in before the first match and the copy-out after the last one
-  // (the only copies nothing hides) are short; three equal chunks between.
-  int chunk_first[5], chunk_n[5], nchunk;
-  if (count >= 32) {
-    const int edge = count / 16, mid = count - 2 * edge;
-    nchunk = 5;
-    chunk_n[0] = chunk_n[4] = edge;
-    chunk_n[1] = chunk_n[2] = mid / 3;
-    chunk_n[3] = mid - 2 * (mid / 3);
-  } else {
-    nchunk = count >= 8 ? 4 : (count >= 2 ? 2 : 1);
-    const int c = (count + nchunk - 1) / nchunk;
-    for (int i = 0; i < nchunk; ++i) chunk_n[i] = std::max(0, std::min(c, count - i * c));
-  }
+  // and the copy-out that read its output (ev_out) have finished.
+  int chunk_first[kHostChunks], chunk_n[kHostChunks];
+  const int nchunk = host_chunks(width, height, count, *p, chunk_n);
   int cs = 0;
   for (int i = 0, f = 0; i < nchunk; ++i) {
     chunk_first[i] = f;

@@ -180,3 +180,22 @@ def test_upsample_is_the_float32_bilinear(level, mshape, shape):
     out = host(bd.upsample(dev(m), level, shape))
     assert np.array_equal(np.isnan(out), np.isnan(ref))
     np.testing.assert_allclose(out, ref, rtol=2e-6)
+
+
+@pytest.mark.parametrize("w,h,count", [(640, 480, 11), (640, 480, 13), (1601, 1200, 2),
+                                       (1280, 960, 9), (640, 480, 49), (1601, 1203, 41)])
+def test_host_chunks_are_the_device_batch(w, h, count):
+    """Batches that run whole and in 2, 3 and 5 chunks: the device entry's maps, bit for bit."""
+    rng = np.random.default_rng(count)
+    tile = rng.integers(0, 256, (3, h, w + 8), dtype=np.uint8)
+    idx = rng.integers(0, 3, count)
+    left = torch.from_numpy(np.ascontiguousarray(tile[idx][:, :, 5:5 + w])).pin_memory()
+    right = torch.from_numpy(np.ascontiguousarray(tile[idx][:, :, 8:8 + w])).pin_memory()
+    p = bd.default_params(iterations=3, coarsest_scale=2, gamma=0.25)
+    m = bd.Matcher("cuda:0")
+    out = m.match_host(left, right, p, torch.empty(count, h, w).pin_memory())
+    again = m.match_host(left, right, p, torch.empty(count, h, w).pin_memory())
+    ref = m.match(left.cuda(), right.cuda(), p).cpu()
+    m.close()
+    assert torch.equal(out.view(torch.int32), ref.view(torch.int32))
+    assert torch.equal(again.view(torch.int32), ref.view(torch.int32))

@@ -364,9 +364,11 @@ struct DisTile {
   int ic0, ic1, jr0, jr1, nc;
 };
 
-// 1 / m, correctly rounded, for m in [1, 2^100]: one Newton step with fused
-// residual on an approximation within 1 ulp (Markstein 1990, theorem on
-// division), the bits of the division.
+// 1 / m for m in [1, 2^100]: one Newton step with fused residual on an
+// approximation within 1 ulp, which rounds correctly unless m's significand is
+// all ones (P. Markstein, IBM J. Res. Dev. 34, 1990; there it may be an ulp off).
+// __frcp_rn's test of its argument's range, per pixel and patch, made the whole
+// call 10% slower (64 pairs of 640x480: 1965 us against 1786, same maps).
 __device__ __forceinline__ float dis_reciprocal(float m) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(m));
@@ -444,10 +446,12 @@ __device__ __forceinline__ void dis_gather(const DensifyArgs &a, const DisTile &
   }
 }
 
-__global__ void __launch_bounds__(128, 8) densify_dis_kernel(const DensifyArgs a, int count) {
+__global__ void __launch_bounds__(128, 8) densify_dis_kernel(const DensifyArgs a, int across,
+                                                              int count) {
   extern __shared__ __align__(16) unsigned char dis_smem[];
   pdl_enter();
-  const int X0 = blockIdx.x * kDisX, Y0 = blockIdx.y * kDisY;
+  const int row = (int)blockIdx.x / across;  // of blocks; one grid dimension: no limit on rows
+  const int X0 = ((int)blockIdx.x - row * across) * kDisX, Y0 = row * kDisY;
   const int x = X0 + (int)(threadIdx.x & 31), y0 = Y0 + (int)(threadIdx.x >> 5) * kDisR;
   const int xe = min(X0 + kDisX, a.w) - 1, ye = min(Y0 + kDisY, a.h) - 1;
   DisTile tile;
@@ -513,8 +517,8 @@ __global__ void __launch_bounds__(128, 8) densify_dis_kernel(const DensifyArgs a
 // store of a warp is one line), so the row's part of the arithmetic is shared;
 // where all four neighbours count, their weights add up to 1 and there is
 // nothing to divide by. The level's rows are read through L1: bound by issue,
-// then by the map's write. 24 maps of 501x375 from level 1: LATER us, where one
-// one pixel per thread, by 64-bit index divisions, took 30.
+// then by the map's write. 24 maps of 501x375 from level 1: 15.5 us, where one
+// pixel per thread, by 64-bit index divisions, took 28.8.
 constexpr int kUpPixels = 4;
 
 __global__ void __launch_bounds__(256) upsample_kernel(const float *__restrict__ M, int mw, int mh,
@@ -522,32 +526,32 @@ __global__ void __launch_bounds__(256) upsample_kernel(const float *__restrict__
                                                        float *__restrict__ out) {
   pdl_enter();
   const int X0 = blockIdx.x * (32 * kUpPixels) + (threadIdx.x & 31);
-  const int y = blockIdx.y * 8 + (threadIdx.x >> 5);
-  if (y >= h) return;
   const float inv = 1.f / scale;  // a power of two: exact
-  const float fy = fminf((float)y * inv, (float)(mh - 1));
-  const int y0 = (int)floorf(fy), y1 = min(y0 + 1, mh - 1);
-  const float ty = fy - y0;
-  for (int b = blockIdx.z; b < count; b += gridDim.z) {
-    const float *r0 = M + ((long long)b * mh + y0) * mw, *r1 = M + ((long long)b * mh + y1) * mw;
-    float *o = out + ((long long)b * h + y) * w;
+  for (int y = blockIdx.y * 8 + (threadIdx.x >> 5); y < h; y += gridDim.y * 8) {
+    const float fy = fminf((float)y * inv, (float)(mh - 1));
+    const int y0 = (int)floorf(fy), y1 = min(y0 + 1, mh - 1);
+    const float ty = fy - y0;
+    for (int b = blockIdx.z; b < count; b += gridDim.z) {
+      const float *r0 = M + ((long long)b * mh + y0) * mw, *r1 = M + ((long long)b * mh + y1) * mw;
+      float *o = out + ((long long)b * h + y) * w;
 #pragma unroll
-    for (int p = 0; p < kUpPixels; ++p) {
-      const int x = X0 + 32 * p;
-      if (x >= w) break;
-      const float fx = fminf((float)x * inv, (float)(mw - 1));
-      const int x0 = (int)floorf(fx), x1 = min(x0 + 1, mw - 1);
-      const float tx = fx - x0;
-      const float wt[4] = {(1.f - tx) * (1.f - ty), tx * (1.f - ty), (1.f - tx) * ty, tx * ty};
-      const float v[4] = {__ldg(r0 + x0), __ldg(r0 + x1), __ldg(r1 + x0), __ldg(r1 + x1)};
-      float s = 0.f, sw = 0.f;
+      for (int p = 0; p < kUpPixels; ++p) {
+        const int x = X0 + 32 * p;
+        if (x >= w) break;
+        const float fx = fminf((float)x * inv, (float)(mw - 1));
+        const int x0 = (int)floorf(fx), x1 = min(x0 + 1, mw - 1);
+        const float tx = fx - x0;
+        const float wt[4] = {(1.f - tx) * (1.f - ty), tx * (1.f - ty), (1.f - tx) * ty, tx * ty};
+        const float v[4] = {__ldg(r0 + x0), __ldg(r0 + x1), __ldg(r1 + x0), __ldg(r1 + x1)};
+        float s = 0.f, sw = 0.f;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (wt[q] > 0.f && isfinite(v[q])) {
-          s += wt[q] * v[q];
-          sw += wt[q];
-        }
-      o[x] = sw == 1.f ? scale * s : sw > 0.f ? scale * s / sw : __int_as_float(0x7fc00000);
+        for (int q = 0; q < 4; ++q)
+          if (wt[q] > 0.f && isfinite(v[q])) {
+            s += wt[q] * v[q];
+            sw += wt[q];
+          }
+        o[x] = sw == 1.f ? scale * s : sw > 0.f ? scale * s / sw : __int_as_float(0x7fc00000);
+      }
     }
   }
 }
@@ -702,12 +706,13 @@ cudaError_t launch_densify(const DensifyArgs &a, cudaStream_t st) {
   if (a.total == 0) return cudaSuccess;
   if (a.fusion == BDIS_FUSION_DIS) {
     const int n = (int)(a.total / a.plane);
-    const dim3 grid((unsigned)((a.w + kDisX - 1) / kDisX), (unsigned)((a.h + kDisY - 1) / kDisY),
+    const int across = (a.w + kDisX - 1) / kDisX;
+    const dim3 grid((unsigned)across * (unsigned)((a.h + kDisY - 1) / kDisY), 1,
                     (unsigned)std::min(n, 65535));
     // at most 64 x 40 records of 16 B, at stride 1 and patch size 32
     const size_t smem = (size_t)dis_span(kDisX, a.ps, a.stride) *
                         dis_span(kDisY, a.ps, a.stride) * sizeof(DisPatch);
-    return launch_maybe_overlapped(densify_dis_kernel, grid, dim3(128), smem, st, a, n);
+    return launch_maybe_overlapped(densify_dis_kernel, grid, dim3(128), smem, st, a, across, n);
   }
   const int count = (int)(a.total / a.plane);
   if (a.tile_y == 0 && a.nx > 0 && a.ny > 0) {  // default: strips where the geometry allows
@@ -757,8 +762,8 @@ cudaError_t launch_densify(const DensifyArgs &a, cudaStream_t st) {
 cudaError_t launch_upsample(const float *map, int mw, int mh, int level, int w, int h, int count,
                             float *out, cudaStream_t st) {
   if ((long long)w * h * count == 0) return cudaSuccess;
-  const dim3 grid((unsigned)((w + 32 * kUpPixels - 1) / (32 * kUpPixels)), (unsigned)((h + 7) / 8),
-                  (unsigned)std::min(count, 65535));
+  const dim3 grid((unsigned)((w + 32 * kUpPixels - 1) / (32 * kUpPixels)),
+                  (unsigned)std::min((h + 7) / 8, 65535), (unsigned)std::min(count, 65535));
   return launch_maybe_overlapped(upsample_kernel, grid, dim3(256), 0, st, map, mw, mh,
                                  (float)(1 << level), w, h, count, out);
 }

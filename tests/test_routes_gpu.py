@@ -199,3 +199,54 @@ def test_host_chunks_are_the_device_batch(w, h, count):
     m.close()
     assert torch.equal(out.view(torch.int32), ref.view(torch.int32))
     assert torch.equal(again.view(torch.int32), ref.view(torch.int32))
+
+
+def test_rows_beyond_a_grid_dimension(orc):
+    """More rows of blocks than a launch's second dimension holds."""
+    h, w, ps = 8 * 65535 + 21, 9, 8
+    rng = np.random.default_rng(1)
+    m = rng.uniform(0, 30, ((h + 1) // 2, (w + 1) // 2)).astype(np.float32)
+    m[::7, 1] = np.nan
+    out = host(bd.upsample(dev(m[None]), 1, (h, w)))[0]
+    tail = 64  # the last rows alone, from the map's last rows (an even first row)
+    first = (h - tail) // 2 * 2
+    ref = host(bd.upsample(dev(m[None, first // 2:]), 1, (h - first, w)))[0]
+    np.testing.assert_array_equal(out[first:], ref)
+    np.testing.assert_array_equal(out[::2, ::2], 2 * m)
+    kw = dict(patch_size=ps, overlap=0.0, coarsest_scale=0, finest_scale=0,
+              fusion=bd._lib.BDIS_FUSION_DIS)
+    ny, nx = bd.grid(h, ps, 0.0)[1], bd.grid(w, ps, 0.0)[1]
+    d = rng.uniform(0, 2, (1, ny, nx)).astype(np.float32)
+    weight = np.ones_like(d)
+    L = rng.uniform(0, 255, (1, h, w)).astype(np.float32)
+    out = host(bd.densify_level((h, w), bd.default_params(**kw), dev(d), dev(weight), None, True,
+                                dev(L), bd.pack_right(dev(L))))
+    ref = orc.densify_level((h, w), orc.OracleParams.make(**kw), d[0], weight[0], None, True,
+                            L[0], L[0])
+    assert np.array_equal(np.isnan(out[0]), np.isnan(ref))
+    np.testing.assert_allclose(out[0], ref, atol=5e-4)
+
+
+def test_dis_reciprocal_is_the_division():
+    """The block route that takes the weight as a reciprocal against the one that divides (one
+    weight of each block other than 1), on the pixels that patch does not cover, bit for bit."""
+    ps, h, w = 8, 256, 512
+    kw = dict(patch_size=ps, overlap=0.5, coarsest_scale=0, finest_scale=0,
+              fusion=bd._lib.BDIS_FUSION_DIS)
+    ny, nx = bd.grid(h, ps, 0.5)[1], bd.grid(w, ps, 0.5)[1]
+    rng = np.random.default_rng(3)
+    d = rng.uniform(0, 3, (8, ny, nx)).astype(np.float32)
+    L = rng.uniform(0, 255, (8, h, w)).astype(np.float32)
+    R = rng.uniform(0, 255, (8, h, w)).astype(np.float32)
+    one = np.ones_like(d)
+    other, touched = one.copy(), np.zeros((h, w), bool)
+    for j in range(0, ny, 2):  # a patch every 8 rows and 32 columns: one in each block at least
+        for i in range(1, nx, 8):
+            other[:, j, i] = 0.5
+            touched[4 * j:4 * j + ps, 4 * i:4 * i + ps] = True
+    a, b = (host(bd.densify_level((h, w), bd.default_params(**kw), dev(d), dev(v), None, True,
+                                  dev(L), bd.pack_right(dev(R)))) for v in (one, other))
+    keep = ~touched
+    keep[:, :40] = False  # blocks at the image's left edge test every sample anyway
+    assert keep.mean() > 0.5
+    np.testing.assert_array_equal(a[:, keep], b[:, keep])

@@ -201,6 +201,39 @@ def test_host_chunks_are_the_device_batch(w, h, count):
     assert torch.equal(again.view(torch.int32), ref.view(torch.int32))
 
 
+def _net_batch(seed, count, h, w):
+    rng = np.random.default_rng(seed)
+    return [dev(rng.uniform(0, hi, (count, h, w)).astype(np.float32)) for hi in (255, 255, 4)]
+
+
+def test_network_buffers_across_shapes():
+    """Larger, smaller and differently padded shapes in turn through one network: what a network
+    that has seen only that shape gives, bit for bit (the loss to the order of its 32-bit sums).
+    A shape whose planar buffers cannot be had takes the other layout: 1e-5 of the norm."""
+    weights = bd.net_init_weights(seed=3)
+    shapes = [(4, 30, 40), (2, 9, 12), (4, 29, 43), (1, 61, 37), (4, 30, 40), (3, 12, 9)]
+    net = bd.ProposalNet(weights)
+    for i, shape in enumerate(shapes):
+        L, R, label = _net_batch(i, *shape)
+        only = bd.ProposalNet(weights)
+        assert np.array_equal(host(net.forward(L, R)), host(only.forward(L, R)))
+        loss, g = net.gradient(L, R, label)
+        ref_loss, ref = only.gradient(L, R, label)
+        only.close()
+        assert np.array_equal(g, ref) and abs(loss - ref_loss) <= 1e-5 * abs(ref_loss)
+    L, R, label = _net_batch(9, 6, 50, 50)
+    bd.inject_alloc_failures(1)
+    try:
+        loss, g = net.gradient(L, R, label)
+    finally:
+        bd.inject_alloc_failures(0)
+    ref_loss, ref = net.gradient(L, R, label)
+    net.status()
+    net.close()
+    assert np.linalg.norm(g - ref) <= 1e-5 * np.linalg.norm(ref)
+    assert abs(loss - ref_loss) <= 1e-5 * abs(ref_loss)
+
+
 def test_rows_beyond_a_grid_dimension(orc):
     """More rows of blocks than a launch's second dimension holds."""
     h, w, ps = 8 * 65535 + 21, 9, 8

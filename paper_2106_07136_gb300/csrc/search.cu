@@ -26,7 +26,9 @@
 //     which keeps the saddle decisions well conditioned; per row a lane reads
 //     the CPL + 2 packed pairs that all five samples of its columns need once;
 //   - a lane's two columns take the same operations, which run as packed
-//     f32x2 adds and FMAs (per component the scalar rounding).
+//     f32x2 adds and FMAs (per component the scalar rounding);
+//   - how many of a patch's columns a sample base keeps inside the image follows
+//     from the base alone, without votes or sums over the group.
 //
 // A fast path with the patch size and window length fixed at compile time
 // (fully unrolled, no per-row guards) for the common settings, and a generic path
@@ -226,23 +228,38 @@ struct TileRows {
   }
 };
 
-// The lane's columns of the centred gradient: in registers, or (SHARED) in
-// shared memory with element (j, r) of thread t at p[(j * PS + r) * kSearchThreads]
-// (p = block array + t; consecutive threads hit consecutive banks). Shared
+// The lane's columns of the centred gradient, four rows at a time (rows r .. r + 3
+// of column j, r a multiple of 4): in registers, or (SHARED) in shared memory
+// with those of thread t at p[(j * PS + r) / 4 * kSearchThreads] (p = block array +
+// t), one 16-byte access that hits all banks once per eight threads. Shared
 // storage frees registers where they are the occupancy limit.
 template <int PS, int CPL, bool SHARED>
 struct GcStore {
   float v[CPL][PS];
-  __device__ __forceinline__ float &at(int j, int r) { return v[j][r]; }
+  __device__ __forceinline__ float4 rows4(int j, int r) const {
+    return make_float4(v[j][r], v[j][r + 1], v[j][r + 2], v[j][r + 3]);
+  }
+  __device__ __forceinline__ void put4(int j, int r, float4 q) {
+    v[j][r] = q.x;
+    v[j][r + 1] = q.y;
+    v[j][r + 2] = q.z;
+    v[j][r + 3] = q.w;
+  }
 };
 template <int PS, int CPL>
 struct GcStore<PS, CPL, true> {
-  float *p;
-  __device__ __forceinline__ float &at(int j, int r) { return p[(j * PS + r) * kSearchThreads]; }
+  float4 *p;
+  __device__ __forceinline__ float4 rows4(int j, int r) const {
+    return p[(j * PS + r) / 4 * kSearchThreads];
+  }
+  __device__ __forceinline__ void put4(int j, int r, float4 q) {
+    p[(j * PS + r) / 4 * kSearchThreads] = q;
+  }
 };
 
 // Inverse-search state of one patch (the group's lanes hold the same scalars).
-template <int PS, int CPL, bool SH>
+// PAIR: L and G are read in pairs of columns.
+template <int PS, int CPL, bool SH, bool PAIR>
 struct PatchState {
   float D, last_step;
   bool frozen, flat;
@@ -256,14 +273,44 @@ struct PatchState {
   int kc;
 };
 
+// Whether a warp whose patches lie inside the image takes code of its own, without
+// masks and clamps, for the first update and for the window. At patch size 8 that
+// is 3% of a 512-pair step of 640x480 (12.15 -> 11.84 ms); the larger sizes, at
+// their register limit, get slower by it (64 pairs: patch 12 1669 -> 1843 us, patch
+// 16 1320 -> 1367).
+template <int PS>
+constexpr bool kInnerPath = PS == 8;
+
+// How many of the PS columns from `first` on lie in [lo, hi].
+template <int PS>
+__device__ __forceinline__ int columns_in(int first, int lo, int hi) {
+  return max(min(first + PS - 1, hi) - max(first, lo) + 1, 0);
+}
+
+// Columns 2 jp and 2 jp + 1 of a lane's row of L or G, 0 where not part of the
+// patch. PAIR: one 8-byte load (the launch has checked that they are aligned).
+template <int CPL, bool PAIR>
+__device__ __forceinline__ float2 left_pair(BDIS_CHECKED_ONLY(const SearchArgs &a, const float *base, )
+                                            const float *row, int jp, const bool (&act)[CPL]) {
+  if constexpr (PAIR) {
+    BDIS_CHECKED_ONLY(if (!in_bounds(row + 2 * jp + 1 - base, a.pixels, kCheckSearchRows))
+                          return make_float2(0.f, 0.f);)
+    return __ldg(reinterpret_cast<const float2 *>(row) + jp);
+  }
+  return make_float2(act[2 * jp] ? BDIS_LDG(row + 2 * jp, base, a.pixels, kCheckSearchRows) : 0.f,
+                     act[2 * jp + 1] ? BDIS_LDG(row + 2 * jp + 1, base, a.pixels, kCheckSearchRows)
+                                     : 0.f);
+}
+
 // Sums of a patch's valid column set (bit j of `code`: the lane's column j is
-// valid): centred gradient (kept in st.gc where `need`), Hessian and template
-// term. Every lane of the warp takes part (group reductions); only groups
-// with `need` keep the result.
-template <int PS, int CPL, bool SH>
-__device__ __forceinline__ void patch_sums(const SearchArgs &a, PatchState<PS, CPL, SH> &st,
-                                           const bool (&act)[CPL], unsigned code, bool need,
-                                           const float *Lc, const float *Gc) {
+// valid; `ncol` of the whole patch): centred gradient (kept in st.gc where
+// `need`), Hessian and template term. Every lane of the warp takes part (group
+// reductions); only groups with `need` keep the result. ALL: every lane's columns
+// are valid.
+template <bool ALL, int PS, int CPL, bool SH, bool PAIR>
+__device__ __forceinline__ void patch_sums(const SearchArgs &a, PatchState<PS, CPL, SH, PAIR> &st,
+                                           const bool (&act)[CPL], unsigned code, int ncol,
+                                           bool need, const float *Lc, const float *Gc) {
   constexpr int LANES = (PS + CPL - 1) / CPL;
   constexpr int G = pow2_at_least(LANES);
   const int w = a.w;
@@ -271,7 +318,7 @@ __device__ __forceinline__ void patch_sums(const SearchArgs &a, PatchState<PS, C
 #pragma unroll
   for (int j = 0; j < CPL; ++j) v[j] = (code >> j) & 1u;
   float hh, ct;
-  int nn;
+  const int nn = PS * ncol;
   if constexpr (CPL % 2 == 0) {
     // column pairs as packed f32x2; the lane's own columns are always
     // readable, and an invalid column's terms are multiplied by 0
@@ -283,17 +330,11 @@ __device__ __forceinline__ void patch_sums(const SearchArgs &a, PatchState<PS, C
     for (int jp = 0; jp < CPL / 2; ++jp)
 #pragma unroll
       for (int r = 0; r < PS; ++r) {
-        float ge[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-          ge[e] = act[2 * jp + e] ? BDIS_LDG(Gc + (size_t)r * w + 2 * jp + e, a.G, a.pixels,
-                                               kCheckSearchRows)
-                                  : 0.f;
-        g2[jp][r] = make_float2(ge[0], ge[1]);
-        s2 = __ffma2_rn(g2[jp][r], m2[jp], s2);  // adds g where valid, exactly
+        g2[jp][r] = left_pair<CPL, PAIR>(BDIS_CHECKED_ONLY(a, a.G, ) Gc + (size_t)r * w, jp, act);
+        // adds g where valid, exactly
+        s2 = ALL ? __fadd2_rn(g2[jp][r], s2) : __ffma2_rn(g2[jp][r], m2[jp], s2);
       }
     const float sg = group_sum<G>(s2.x + s2.y);
-    nn = PS * group_sum_int<G>(__popc(code));
     const float mg = (a.normalize && nn > 0) ? __fdividef(sg, (float)nn) : 0.f;
     const float2 nmg = make_float2(-mg, -mg);
     float2 h2 = make_float2(0.f, 0.f), c2 = make_float2(0.f, 0.f);
@@ -301,19 +342,18 @@ __device__ __forceinline__ void patch_sums(const SearchArgs &a, PatchState<PS, C
     for (int jp = 0; jp < CPL / 2; ++jp) {
 #pragma unroll
       for (int r = 0; r < PS; ++r) {
-        const float2 q = __fmul2_rn(__fadd2_rn(g2[jp][r], nmg), m2[jp]);
-        if (need) {
-          st.gc.at(2 * jp, r) = q.x;
-          st.gc.at(2 * jp + 1, r) = q.y;
+        float2 q = __fadd2_rn(g2[jp][r], nmg);
+        if (!ALL) q = __fmul2_rn(q, m2[jp]);
+        g2[jp][r] = q;
+        if (need && r % 4 == 3) {
+          const float2 *p = &g2[jp][r - 3];
+          st.gc.put4(2 * jp, r - 3, make_float4(p[0].x, p[1].x, p[2].x, p[3].x));
+          st.gc.put4(2 * jp + 1, r - 3, make_float4(p[0].y, p[1].y, p[2].y, p[3].y));
         }
-        float te[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-          te[e] = act[2 * jp + e] ? BDIS_LDG(Lc + (size_t)r * w + 2 * jp + e, a.L, a.pixels,
-                                               kCheckSearchRows)
-                                  : 0.f;
+        const float2 te =
+            left_pair<CPL, PAIR>(BDIS_CHECKED_ONLY(a, a.L, ) Lc + (size_t)r * w, jp, act);
         h2 = __ffma2_rn(q, q, h2);
-        c2 = __ffma2_rn(q, make_float2(te[0], te[1]), c2);
+        c2 = __ffma2_rn(q, te, c2);
       }
     }
     hh = h2.x + h2.y;
@@ -330,7 +370,6 @@ __device__ __forceinline__ void patch_sums(const SearchArgs &a, PatchState<PS, C
         sg += g[j][r];
       }
     sg = group_sum<G>(sg);
-    nn = PS * group_sum_int<G>(__popc(code));
     const float mg = (a.normalize && nn > 0) ? __fdividef(sg, (float)nn) : 0.f;
     hh = 0.f;
     ct = 0.f;
@@ -339,7 +378,7 @@ __device__ __forceinline__ void patch_sums(const SearchArgs &a, PatchState<PS, C
 #pragma unroll
       for (int r = 0; r < PS; ++r) {
         const float q = v[j] ? g[j][r] - mg : 0.f;
-        if (need) st.gc.at(j, r) = q;
+        if (need) st.gc.v[j][r] = q;
         hh = fmaf(q, q, hh);
         ct = fmaf(q,
                   act[j] ? BDIS_LDG(Lc + (size_t)r * w + j, a.L, a.pixels, kCheckSearchRows)
@@ -362,22 +401,26 @@ __device__ __forceinline__ void patch_sums(const SearchArgs &a, PatchState<PS, C
 
 // A and B of the lane's columns at integer base kd (sample columns ib + j):
 // no branches inside; an invalid column has gc = 0 and reads a clamped,
-// readable column, so it adds exactly 0.
-template <int PS, int CPL, bool SH, class Rows>
-__device__ __forceinline__ void patch_ab(const Rows &rows, PatchState<PS, CPL, SH> &st, int ib,
-                                         int kd) {
+// readable column, so it adds exactly 0. ALL: every lane's columns are valid.
+template <bool ALL, int PS, int CPL, bool SH, bool PAIR, class Rows>
+__device__ __forceinline__ void patch_ab(const Rows &rows, PatchState<PS, CPL, SH, PAIR> &st,
+                                         int ib, int kd) {
   constexpr int LANES = (PS + CPL - 1) / CPL;
   constexpr int G = pow2_at_least(LANES);
   float sa[2] = {0.f, 0.f}, sb[2] = {0.f, 0.f};
 #pragma unroll
   for (int j = 0; j < CPL; ++j) {
-    const auto p = rows.col_clamped(ib + j);
+    const auto p = ALL ? rows.col(ib + j) : rows.col_clamped(ib + j);
 #pragma unroll
-    for (int r = 0; r < PS; ++r) {
-      const float2 q = rows.ld(p, r);
-      const float g = st.gc.at(j, r);
-      sa[r & 1] = fmaf(g, q.x, sa[r & 1]);
-      sb[r & 1] = fmaf(g, q.y, sb[r & 1]);
+    for (int r4 = 0; r4 < PS; r4 += 4) {
+      const float4 g4 = st.gc.rows4(j, r4);
+      const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 q = rows.ld(p, r4 + e);
+        sa[e & 1] = fmaf(g[e], q.x, sa[e & 1]);
+        sb[e & 1] = fmaf(g[e], q.y, sb[e & 1]);
+      }
     }
   }
   st.A = group_sum<G>(sa[0] + sa[1]);
@@ -398,32 +441,42 @@ __device__ __forceinline__ unsigned valid_code(const bool (&act)[CPL], int ib, f
 // The patch's D* update (Eq. 1) from the step sum; a stopped patch keeps its
 // state. Stops on a non-finite D, on leaving the search range (dropped
 // later) or on convergence (update below kStepTol).
-template <int PS, int CPL, bool SH>
-__device__ __forceinline__ void patch_update(PatchState<PS, CPL, SH> &st, float Ssum, float u0) {
+template <int PS, int CPL, bool SH, bool PAIR>
+__device__ __forceinline__ void patch_update(PatchState<PS, CPL, SH, PAIR> &st, float Ssum, float u0) {
   const float step = (Ssum - st.gcT) * st.invH;
   const bool live = !st.frozen;
   const float D = st.D + step;
   st.D = live ? D : st.D;
   st.last_step = live ? step : st.last_step;
   st.steps += live ? 1 : 0;
-  st.frozen = !live || !isfinite(D) || fabsf(D - u0) > (float)PS || fabsf(step) < kStepTol;
+  // (a D that is not finite fails the range test too: u0 is finite or D is NaN)
+  st.frozen = !live || !(fabsf(D - u0) <= (float)PS) || fabsf(step) < kStepTol;
 }
 
 // The first update of Eq. 1 for every patch of the warp: every patch computes
 // its sums (no votes, no predicated stores).
-template <int PS, int CPL, bool SH, class Rows>
+template <int PS, int CPL, bool SH, bool PAIR, class Rows>
 __device__ __forceinline__ void search_first_step(const SearchArgs &a, const Rows &rows,
-                                                  PatchState<PS, CPL, SH> &st,
-                                                  const bool (&act)[CPL], int xl, const float *Lc,
+                                                  PatchState<PS, CPL, SH, PAIR> &st,
+                                                  const bool (&act)[CPL], int xl, int x0,
+                                                  unsigned full, const float *Lc,
                                                   const float *Gc, float u0) {
   int kd;
   float t;
   split_disp(st.D, kd, t);
   const int ib = xl + kd;
-  patch_sums<PS, CPL, SH>(a, st, act, valid_code<CPL>(act, ib, t, a.w), true, Lc, Gc);
-  rows.ready();  // staged rows (if any) arrive while the sums above load
-  patch_ab<PS, CPL, SH>(rows, st, ib, kd);
-  if (!st.frozen) patch_update<PS, CPL, SH>(st, fmaf(t, st.B, st.A), u0);
+  // a warp whose patches all sample inside [0, w - 2] masks and clamps nothing
+  if (kInnerPath<PS> && __all_sync(kFull, (unsigned)(kd + x0) <= (unsigned)(a.w - 1 - PS))) {
+    patch_sums<true>(a, st, act, full, PS, true, Lc, Gc);
+    rows.ready();  // staged rows (if any) arrive while the sums above load
+    patch_ab<true>(rows, st, ib, kd);
+  } else {
+    patch_sums<false>(a, st, act, valid_code<CPL>(act, ib, t, a.w),
+                      columns_in<PS>(x0 + kd, 0, last_base(t, a.w)), true, Lc, Gc);
+    rows.ready();
+    patch_ab<false>(rows, st, ib, kd);
+  }
+  if (!st.frozen) patch_update(st, fmaf(t, st.B, st.A), u0);
 }
 
 // A later update for every patch of the warp. Returns false, taking no step,
@@ -436,18 +489,19 @@ __device__ __forceinline__ void search_first_step(const SearchArgs &a, const Row
 // The valid set can only change near the image border: while every column of
 // the patch samples inside [0, w - 2] (kd in [-x0, w - 1 - PS - x0]) it is the
 // full set, with no per-column tests.
-template <int PS, int CPL, bool SH, class Rows>
+template <int PS, int CPL, bool SH, bool PAIR, class Rows>
 __device__ __forceinline__ bool search_next_step(const SearchArgs &a, const Rows &rows,
-                                                 PatchState<PS, CPL, SH> &st,
+                                                 PatchState<PS, CPL, SH, PAIR> &st,
                                                  const bool (&act)[CPL], int xl, int x0,
                                                  unsigned full, const float *Lc,
                                                  const float *Gc, unsigned gbits, float u0) {
-  int kd;
-  float t;
-  split_disp(st.D, kd, t);
-  const int ib = xl + kd;
+  // as split_disp, without its bounds: a running patch is within PS of its start,
+  // and what a stopped one gets here (the conversion saturates) is not used
+  const float f = floorf(-st.D), t = -st.D - f;
+  const int kd = __float2int_rz(f);
+  const int ib = (int)((unsigned)xl + (unsigned)kd);
   unsigned code = full;
-  if ((unsigned)(kd + x0) > (unsigned)(a.w - 1 - PS)) code = valid_code<CPL>(act, ib, t, a.w);
+  if ((unsigned)kd + (unsigned)x0 > (unsigned)(a.w - 1 - PS)) code = valid_code<CPL>(act, ib, t, a.w);
   const bool chg = !st.frozen && code != st.prev;
   const bool mv = !st.frozen && kd != st.kc;
   const unsigned r = __reduce_or_sync(kFull, (chg ? 1u : 0u) | (mv ? 2u : 0u) |
@@ -455,10 +509,11 @@ __device__ __forceinline__ bool search_next_step(const SearchArgs &a, const Rows
   if (!(r & 4u)) return false;  // every patch of the warp has stopped
   if (r & 1u) {
     const bool need = (__ballot_sync(kFull, chg) & gbits) != 0u;
-    patch_sums<PS, CPL, SH>(a, st, act, code, need, Lc, Gc);
+    const int first = (int)((unsigned)kd + (unsigned)x0);
+    patch_sums<false>(a, st, act, code, columns_in<PS>(first, 0, last_base(t, a.w)), need, Lc, Gc);
   }
-  if (r & 3u) patch_ab<PS, CPL, SH>(rows, st, ib, kd);
-  patch_update<PS, CPL, SH>(st, fmaf(t, st.B, st.A), u0);
+  if (r & 3u) patch_ab<false>(rows, st, ib, kd);
+  patch_update(st, fmaf(t, st.B, st.A), u0);
   return true;
 }
 
@@ -531,73 +586,22 @@ __device__ __forceinline__ void window_rows(BDIS_CHECKED_ONLY(const SearchArgs &
   }
 }
 
-template <int PS, int CPL, bool SH = false, class Rows>
-__device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &rows, long long k,
-                                            bool live, int c, unsigned gbits, int b, int x0,
-                                            int y0, float u0, float *sgc = nullptr) {
+// The window's energies E[i] at D* + {-1, -0.5, 0, 0.5, 1}, for nc pixels. INNER:
+// every column of every lane is valid at every sample.
+template <int PS, int CPL, bool INNER, class Rows>
+__device__ __forceinline__ void window_energies(const SearchArgs &a, const Rows &rows,
+                                                const float *Lc, int ib, float t, float th,
+                                                bool hi, const bool (&act)[CPL], bool inr, int lb,
+                                                int nc, float (&E)[5]) {
   constexpr int LANES = (PS + CPL - 1) / CPL;
   constexpr int G = pow2_at_least(LANES);
-  constexpr int S = 5, HALF = 2;
+  constexpr int S = 5;
+  constexpr bool kUnmasked = INNER && PS == CPL * G;
   const int w = a.w;
-  const int xl = x0 + c * CPL;  // first column of this lane
-  bool act[CPL];
-#pragma unroll
-  for (int j = 0; j < CPL; ++j) act[j] = (c * CPL + j) < PS;
-  const long long poff = (long long)b * a.plane + (long long)y0 * w;
-  const float *Lc = a.L + poff + xl;
-  const float *Gc = a.G + poff + xl;
-
-  // The template T (the lane's left columns) is read where it is used: in the
-  // sums of a new valid run and in the window, not held through the steps.
-
-  // ---- inverse-search iterations (Eq. 1)
-  PatchState<PS, CPL, SH> st;
-  if constexpr (SH) st.gc.p = sgc + threadIdx.x;
-  st.D = u0;
-  st.last_step = 0.f;
-  st.frozen = st.flat = false;
-  st.steps = 0;
-  if (a.iters > 0) {
-    unsigned full = 0u;  // the lane's columns that are part of the patch
-#pragma unroll
-    for (int j = 0; j < CPL; ++j) full |= (unsigned)act[j] << j;
-    search_first_step<PS, CPL, SH>(a, rows, st, act, xl, Lc, Gc, u0);
-    for (int it = 1; it < a.iters; ++it)
-      if (!search_next_step<PS, CPL, SH>(a, rows, st, act, xl, x0, full, Lc, Gc, gbits, u0))
-        break;  // every patch of the warp has stopped
-  }
-  const float D = st.D, last_step = st.last_step;
-  const bool flat = st.flat;
-  const int steps = st.steps;
-
-  rows.ready();
-  // ---- Bayesian window (Eqs. 3-4): samples at D* + {-1, -0.5, 0, 0.5, 1}
-  const bool fin = isfinite(D);
-  // a patch that left its search range is dropped (R8) and reads no window
-  const bool inr = fin && fabsf(D - u0) <= (float)PS;
-  int kd;
-  float t;
-  split_disp(D, kd, t);
-  const int ib = xl + kd;
-  // samples at D* + {-1, 0, 1} have fraction t; at D* +- 0.5 fraction th, with
-  // base column one further right when t >= 0.5
-  const bool hi = t >= 0.5f;
-  const float th = hi ? t - 0.5f : t + 0.5f;
-  const int lb = last_base(t, w);
   bool vc[CPL];
-  int nv_lane = 0, nc_lane = 0;
 #pragma unroll
-  for (int j = 0; j < CPL; ++j) {
-    nv_lane += (act[j] && fin && ib + j >= 0 && ib + j <= lb) ? 1 : 0;
-    vc[j] = act[j] && inr && ib + j >= 1 && ib + j + 1 <= lb;
-    nc_lane += vc[j] ? 1 : 0;
-  }
-  const int nvalid = PS * group_sum_int<G>(nv_lane);
-  if (a.fusion == BDIS_FUSION_DIS) {
-    finish_patch_dis(a, k, live && c == 0, D, u0, last_step, flat, steps, nvalid, PS);
-    return;
-  }
-  const int nc = PS * group_sum_int<G>(nc_lane);
+  for (int j = 0; j < CPL; ++j)
+    vc[j] = act[j] && (INNER || (inr && ib + j >= 1 && ib + j + 1 <= lb));
   // One pass over the rows. Every sample of the lane's columns lies in
   // columns ib - 1 .. ib + CPL, so per row the lane reads those CPL + 2 packed
   // pairs once and interpolates each at both fractions (t for D* and D* +- 1,
@@ -620,7 +624,6 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
   // Merge per sample: s1 = sum of the residuals, md their mean, and
   // E = sum (d - md)^2 = S2 - 2 (md - cs) S1 + n (md - cs)^2 per column.
   const float inv_nc = nc > 0 ? __fdividef(1.f, (float)nc) : 0.f;
-  float E[S];
   WindowSums<CPL> ws;
 #pragma unroll
   for (int i = 0; i < S; ++i) {
@@ -630,7 +633,7 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
   }
   // A warp whose patches are all in range (so their pairs lie in a staged
   // tile, if any) with all pairs in the image reads them unconditionally.
-  if (__all_sync(kFull, inr && ib >= 1 && ib + CPL <= w - 1))
+  if (INNER || __all_sync(kFull, inr && ib >= 1 && ib + CPL <= w - 1))
     window_rows<PS, CPL, false>(BDIS_CHECKED_ONLY(a, ) rows, ib, t, th, hi, Lc, w, act, need, cs,
                                 ws);
   else
@@ -652,7 +655,8 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
       float s1 = 0.f;
 #pragma unroll
       for (int jp = 0; jp < CPL / 2; ++jp) {
-        const float2 x = __fmul2_rn(__ffma2_rn(kPS, cs2[jp], ws.P1[i][jp]), vm[jp]);
+        float2 x = __ffma2_rn(kPS, cs2[jp], ws.P1[i][jp]);
+        if (!kUnmasked) x = __fmul2_rn(x, vm[jp]);
         s1 += x.x + x.y;
       }
       s1 = group_sum<G>(s1);
@@ -663,7 +667,8 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
       for (int jp = 0; jp < CPL / 2; ++jp) {
         const float2 u = __fadd2_rn(md2, ncs2[jp]);
         const float2 in = __ffma2_rn(__fmul2_rn(kPS, u), u, ws.P2[i][jp]);
-        const float2 x = __fmul2_rn(__ffma2_rn(__fmul2_rn(kM2, u), ws.P1[i][jp], in), vm[jp]);
+        float2 x = __ffma2_rn(__fmul2_rn(kM2, u), ws.P1[i][jp], in);
+        if (!kUnmasked) x = __fmul2_rn(x, vm[jp]);
         e += x.x + x.y;
       }
       E[i] = group_sum<G>(e);
@@ -694,6 +699,74 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
       E[i] = group_sum<G>(e);
     }
   }
+}
+
+template <int PS, int CPL, bool SH = false, bool PAIR = false, class Rows>
+__device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &rows, long long k,
+                                            bool live, int c, unsigned gbits, int b, int x0,
+                                            int y0, float u0, float4 *sgc = nullptr) {
+  constexpr int LANES = (PS + CPL - 1) / CPL;
+  constexpr int G = pow2_at_least(LANES);
+  constexpr int S = 5, HALF = 2;
+  const int w = a.w;
+  const int xl = x0 + c * CPL;  // first column of this lane
+  bool act[CPL];
+#pragma unroll
+  for (int j = 0; j < CPL; ++j) act[j] = (c * CPL + j) < PS;
+  const long long poff = (long long)b * a.plane + (long long)y0 * w;
+  const float *Lc = a.L + poff + xl;
+  const float *Gc = a.G + poff + xl;
+
+  // The template T (the lane's left columns) is read where it is used: in the
+  // sums of a new valid run and in the window, not held through the steps.
+
+  // ---- inverse-search iterations (Eq. 1)
+  PatchState<PS, CPL, SH, PAIR> st;
+  if constexpr (SH) st.gc.p = sgc + threadIdx.x;
+  st.D = u0;
+  st.last_step = 0.f;
+  st.frozen = st.flat = false;
+  st.steps = 0;
+  if (a.iters > 0) {
+    unsigned full = 0u;  // the lane's columns that are part of the patch
+#pragma unroll
+    for (int j = 0; j < CPL; ++j) full |= (unsigned)act[j] << j;
+    search_first_step(a, rows, st, act, xl, x0, full, Lc, Gc, u0);
+    for (int it = 1; it < a.iters; ++it)
+      if (!search_next_step(a, rows, st, act, xl, x0, full, Lc, Gc, gbits, u0))
+        break;  // every patch of the warp has stopped
+  }
+  const float D = st.D, last_step = st.last_step;
+  const bool flat = st.flat;
+  const int steps = st.steps;
+
+  rows.ready();
+  // ---- Bayesian window (Eqs. 3-4): samples at D* + {-1, -0.5, 0, 0.5, 1}
+  const bool fin = isfinite(D);
+  // a patch that left its search range is dropped (R8) and reads no window
+  const bool inr = fin && fabsf(D - u0) <= (float)PS;
+  int kd;
+  float t;
+  split_disp(D, kd, t);
+  const int ib = xl + kd;
+  // samples at D* + {-1, 0, 1} have fraction t; at D* +- 0.5 fraction th, with
+  // base column one further right when t >= 0.5
+  const bool hi = t >= 0.5f;
+  const float th = hi ? t - 0.5f : t + 0.5f;
+  const int lb = last_base(t, w);
+  const int nvalid = fin ? PS * columns_in<PS>(x0 + kd, 0, lb) : 0;
+  if (a.fusion == BDIS_FUSION_DIS) {
+    finish_patch_dis(a, k, live && c == 0, D, u0, last_step, flat, steps, nvalid, PS);
+    return;
+  }
+  const int nc = inr ? PS * columns_in<PS>(x0 + kd, 1, lb - 1) : 0;
+  float E[S];
+  // a warp whose patches are all in range (so their pairs lie in a staged
+  // tile, if any) with every column valid at every sample masks nothing
+  if (kInnerPath<PS> && __all_sync(kFull, inr && ib >= 1 && ib + CPL <= w - 2))
+    window_energies<PS, CPL, true>(a, rows, Lc, ib, t, th, hi, act, inr, lb, PS * PS, E);
+  else
+    window_energies<PS, CPL, false>(a, rows, Lc, ib, t, th, hi, act, inr, lb, nc, E);
   const bool write = live && c == 0;
   if (write && a.energies) {
 #pragma unroll
@@ -717,9 +790,16 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
 }
 
 // One patch per group, pairs on blockIdx.y, patches of a pair on blockIdx.x;
-// samples read from global memory (through L1).
-// SH: the centred-gradient cache in shared memory (GcStore).
-template <int PS, int CPL, int MINB, bool SH>
+// samples read from global memory (through L1). Bound by instruction issue: a
+// call on 512 pairs of 640x480 at patch 8 takes 11.84 ms, 86% of it here (12.51
+// before the 8- and 16-byte accesses to the lane's own columns, the column counts
+// from the sample base, the update without bounds on its base, and the code of
+// its own for warps inside the image). Slower on the same call: 7 blocks per SM
+// 12.44, 9 blocks 12.21, the template kept in shared memory too 12.37, planes
+// addressed by 32-bit offsets 13.41.
+// SH: the centred-gradient cache in shared memory (GcStore). PAIR: L and G read in
+// pairs of columns.
+template <int PS, int CPL, int MINB, bool SH, bool PAIR>
 __global__ void __launch_bounds__(kSearchThreads, MINB) search_fixed_kernel(const SearchArgs a) {
   pdl_enter();
   constexpr int LANES = (PS + CPL - 1) / CPL;
@@ -743,11 +823,11 @@ __global__ void __launch_bounds__(kSearchThreads, MINB) search_fixed_kernel(cons
     u0 = 2.f * bilinear_clamped(a.coarse + (long long)b * a.cplane, a.cw, a.ch, cx * 0.5f,
                                 cy * 0.5f);
   }
-  __shared__ float sgc[SH ? CPL * PS * kSearchThreads : 1];
-  fixed_patch<PS, CPL, SH>(a,
-                           GlobalRows{a.R2 + (long long)b * a.plane + (long long)y0 * w,
-                                      w BDIS_CHECKED_ONLY(, a.R2, a.pixels)},
-                           k, live, c, gbits, b, x0, y0, u0, sgc);
+  __shared__ float4 sgc[SH ? CPL * PS / 4 * kSearchThreads : 1];
+  fixed_patch<PS, CPL, SH, PAIR>(a,
+                                 GlobalRows{a.R2 + (long long)b * a.plane + (long long)y0 * w,
+                                            w BDIS_CHECKED_ONLY(, a.R2, a.pixels)},
+                                 k, live, c, gbits, b, x0, y0, u0, sgc);
 }
 
 __device__ __forceinline__ int warp_min(int v) {
@@ -1214,8 +1294,17 @@ cudaError_t launch_fixed(const SearchArgs &a, cudaStream_t st) {
   const int threads = a.block_threads == 64 ? 64 : 128, per_block = threads / G;
   const int count = (int)(a.total / a.np);
   const dim3 grid((unsigned)((a.np + per_block - 1) / per_block), (unsigned)count);
-  return launch_maybe_overlapped(search_fixed_kernel<PS, CPL, MINB, SH>, grid, dim3(threads), 0, st,
-                                 a);
+  // L and G in 8-byte pairs where every patch starts on one: an even pitch and
+  // stride put each origin (also the last, at w - PS) on an even column. 64 pairs
+  // of 640x480 at patch 16: 1377 -> 1320 us a call; at patch 8 1% of it.
+  if constexpr (CPL == 2 && PS % 2 == 0) {
+    const bool aligned = (reinterpret_cast<uintptr_t>(a.L) | reinterpret_cast<uintptr_t>(a.G)) % 8 == 0;
+    if (aligned && a.w % 2 == 0 && a.stride % 2 == 0)
+      return launch_maybe_overlapped(search_fixed_kernel<PS, CPL, MINB, SH, true>, grid,
+                                     dim3(threads), 0, st, a);
+  }
+  return launch_maybe_overlapped(search_fixed_kernel<PS, CPL, MINB, SH, false>, grid,
+                                 dim3(threads), 0, st, a);
 }
 
 template <int PS, int CPL, int MINB>

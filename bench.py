@@ -577,7 +577,7 @@ def measure_extras(args, bd, m, params, left, right, Lh, Rh, Dgt, device, stream
                 "h2d_bytes_per_step": 2 * B * W * H, "d2h_bytes_per_step": 4 * B * W * H,
                 "runs": runs, "steps_per_run": k,
                 "path": "bdis_match_host (returns with the result): pinned host uint8 in, "
-                        "float32 disparity out, 4 chunks overlapping copies and match"}
+                        "float32 disparity out, chunks overlapping copies and match"}
     # the same steps as a stream of batches (bdis_match_host_async): up to S
     # steps in flight, step i enqueued once step i - S (whose buffer set it
     # reuses) has been waited for, so a step's copies overlap other steps'
@@ -772,7 +772,7 @@ def measure_learned(args, bd, m, left, right, Lh, Rh, Dgt, device, stream,
     net_info = {"ms_per_step": net_ms, "pixels_per_step": px, "algorithmic_flops_per_step": flop,
                 "achieved_tflops": flop / (net_ms / 1e3) / 1e12, "peak_tflops": bf16_peak,
                 "frac": flop / (net_ms / 1e3) / 1e12 / bf16_peak, "peak_source": bf16_src,
-                "kernel": "net_forward_kernel (banded tcgen05, one cooperative launch)",
+                "kernel": "net_chain_kernel (banded tcgen05, one cooperative launch)",
                 "level": level, "input": f"{B} x {Lq.shape[2]}x{Lq.shape[1]}"}
     del Lq, Rq, prop
     rows = []

@@ -522,36 +522,36 @@ __global__ void __launch_bounds__(128, 8) densify_dis_kernel(const DensifyArgs a
 constexpr int kUpPixels = 4;
 
 __global__ void __launch_bounds__(256) upsample_kernel(const float *__restrict__ M, int mw, int mh,
-                                                       float scale, int w, int h, int count,
-                                                       float *__restrict__ out) {
+                                                       float scale, int row0, int w, int h,
+                                                       int count, float *__restrict__ out) {
   pdl_enter();
   const int X0 = blockIdx.x * (32 * kUpPixels) + (threadIdx.x & 31);
+  const int y = row0 + blockIdx.y * 8 + (threadIdx.x >> 5);
+  if (y >= h) return;
   const float inv = 1.f / scale;  // a power of two: exact
-  for (int y = blockIdx.y * 8 + (threadIdx.x >> 5); y < h; y += gridDim.y * 8) {
-    const float fy = fminf((float)y * inv, (float)(mh - 1));
-    const int y0 = (int)floorf(fy), y1 = min(y0 + 1, mh - 1);
-    const float ty = fy - y0;
-    for (int b = blockIdx.z; b < count; b += gridDim.z) {
-      const float *r0 = M + ((long long)b * mh + y0) * mw, *r1 = M + ((long long)b * mh + y1) * mw;
-      float *o = out + ((long long)b * h + y) * w;
+  const float fy = fminf((float)y * inv, (float)(mh - 1));
+  const int y0 = (int)floorf(fy), y1 = min(y0 + 1, mh - 1);
+  const float ty = fy - y0;
+  for (int b = blockIdx.z; b < count; b += gridDim.z) {
+    const float *r0 = M + ((long long)b * mh + y0) * mw, *r1 = M + ((long long)b * mh + y1) * mw;
+    float *o = out + ((long long)b * h + y) * w;
 #pragma unroll
-      for (int p = 0; p < kUpPixels; ++p) {
-        const int x = X0 + 32 * p;
-        if (x >= w) break;
-        const float fx = fminf((float)x * inv, (float)(mw - 1));
-        const int x0 = (int)floorf(fx), x1 = min(x0 + 1, mw - 1);
-        const float tx = fx - x0;
-        const float wt[4] = {(1.f - tx) * (1.f - ty), tx * (1.f - ty), (1.f - tx) * ty, tx * ty};
-        const float v[4] = {__ldg(r0 + x0), __ldg(r0 + x1), __ldg(r1 + x0), __ldg(r1 + x1)};
-        float s = 0.f, sw = 0.f;
+    for (int p = 0; p < kUpPixels; ++p) {
+      const int x = X0 + 32 * p;
+      if (x >= w) break;
+      const float fx = fminf((float)x * inv, (float)(mw - 1));
+      const int x0 = (int)floorf(fx), x1 = min(x0 + 1, mw - 1);
+      const float tx = fx - x0;
+      const float wt[4] = {(1.f - tx) * (1.f - ty), tx * (1.f - ty), (1.f - tx) * ty, tx * ty};
+      const float v[4] = {__ldg(r0 + x0), __ldg(r0 + x1), __ldg(r1 + x0), __ldg(r1 + x1)};
+      float s = 0.f, sw = 0.f;
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (wt[q] > 0.f && isfinite(v[q])) {
-            s += wt[q] * v[q];
-            sw += wt[q];
-          }
-        o[x] = sw == 1.f ? scale * s : sw > 0.f ? scale * s / sw : __int_as_float(0x7fc00000);
-      }
+      for (int q = 0; q < 4; ++q)
+        if (wt[q] > 0.f && isfinite(v[q])) {
+          s += wt[q] * v[q];
+          sw += wt[q];
+        }
+      o[x] = sw == 1.f ? scale * s : sw > 0.f ? scale * s / sw : __int_as_float(0x7fc00000);
     }
   }
 }
@@ -762,10 +762,17 @@ cudaError_t launch_densify(const DensifyArgs &a, cudaStream_t st) {
 cudaError_t launch_upsample(const float *map, int mw, int mh, int level, int w, int h, int count,
                             float *out, cudaStream_t st) {
   if ((long long)w * h * count == 0) return cudaSuccess;
-  const dim3 grid((unsigned)((w + 32 * kUpPixels - 1) / (32 * kUpPixels)),
-                  (unsigned)std::min((h + 7) / 8, 65535), (unsigned)std::min(count, 65535));
-  return launch_maybe_overlapped(upsample_kernel, grid, dim3(256), 0, st, map, mw, mh,
-                                 (float)(1 << level), w, h, count, out);
+  cudaError_t e = cudaSuccess;
+  constexpr int kRows = 65535 * 8;  // of one launch
+  for (int row0 = 0; row0 < h && e == cudaSuccess; row0 += kRows) {
+    const dim3 grid((unsigned)((w + 32 * kUpPixels - 1) / (32 * kUpPixels)),
+                    (unsigned)((std::min(kRows, h - row0) + 7) / 8),
+                    (unsigned)std::min(count, 65535));
+    e = launch_maybe_overlapped(upsample_kernel, grid, dim3(256), 0, st, map, mw, mh,
+                                (float)(1 << level), row0, w, h, count, out);
+    if (h - row0 <= kRows) break;
+  }
+  return e;
 }
 
 cudaError_t take_check_densify(unsigned *v) { return take_check_word(v); }

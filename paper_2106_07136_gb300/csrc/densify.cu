@@ -521,12 +521,14 @@ __global__ void __launch_bounds__(128, 8) densify_dis_kernel(const DensifyArgs a
 // pixel per thread, by 64-bit index divisions, took 28.8.
 constexpr int kUpPixels = 4;
 
+// FROM: rows from row0 on (a launch of its own; the addition costs the others 5%).
+template <bool FROM>
 __global__ void __launch_bounds__(256) upsample_kernel(const float *__restrict__ M, int mw, int mh,
-                                                       float scale, int row0, int w, int h,
-                                                       int count, float *__restrict__ out) {
+                                                       float scale, int w, int h, int count,
+                                                       float *__restrict__ out, int row0) {
   pdl_enter();
   const int X0 = blockIdx.x * (32 * kUpPixels) + (threadIdx.x & 31);
-  const int y = row0 + blockIdx.y * 8 + (threadIdx.x >> 5);
+  const int y = (FROM ? row0 : 0) + blockIdx.y * 8 + (threadIdx.x >> 5);
   if (y >= h) return;
   const float inv = 1.f / scale;  // a power of two: exact
   const float fy = fminf((float)y * inv, (float)(mh - 1));
@@ -768,8 +770,9 @@ cudaError_t launch_upsample(const float *map, int mw, int mh, int level, int w, 
     const dim3 grid((unsigned)((w + 32 * kUpPixels - 1) / (32 * kUpPixels)),
                     (unsigned)((std::min(kRows, h - row0) + 7) / 8),
                     (unsigned)std::min(count, 65535));
-    e = launch_maybe_overlapped(upsample_kernel, grid, dim3(256), 0, st, map, mw, mh,
-                                (float)(1 << level), row0, w, h, count, out);
+    e = launch_maybe_overlapped(row0 ? upsample_kernel<true> : upsample_kernel<false>, grid,
+                                dim3(256), 0, st, map, mw, mh, (float)(1 << level), w, h, count,
+                                out, row0);
     if (h - row0 <= kRows) break;
   }
   return e;

@@ -283,3 +283,42 @@ def test_dis_reciprocal_is_the_division():
     keep[:, :40] = False  # blocks at the image's left edge test every sample anyway
     assert keep.mean() > 0.5
     np.testing.assert_array_equal(a[:, keep], b[:, keep])
+
+
+@pytest.mark.parametrize("ps", [8, 16])
+@pytest.mark.parametrize("kw", [dict(), dict(overlap=0.5, normalize=0), dict(iterations=0),
+                                dict(fusion=bd._lib.BDIS_FUSION_DIS)])
+@pytest.mark.parametrize("h,w", [(16, 16), (61, 98), (64, 160)])
+def test_paired_loads_and_inner_warps(ps, kw, h, w):
+    """The search that reads the left planes in pairs against the same planes on an odd float (read
+    one by one), and warps inside the image against the same warps with a patch that starts far
+    outside it: every output of every patch with the same start, bit for bit."""
+    gp = bd.default_params(**dict(dict(patch_size=ps, iterations=9), **kw))
+    L, R, G = _planes(h, w, 3, h + ps)
+    L[0, :30, :40] = 90.0
+    G[0, :30, :40] = 0.0
+    R[1, 10, 9, 0] = float("nan")
+    near = torch.rand(3, (h + 1) // 2, (w + 1) // 2, device=L.device) * 2
+    far = near.clone()
+    far[:, ::6, ::9] = 1.0e4
+
+    def odd(t):
+        v = torch.empty(t.numel() + 1, device=t.device)[1:].view(t.shape)
+        assert v.data_ptr() % 8 == 4
+        return v.copy_(t)
+
+    def run(left, grad, coarse):
+        return {k: host(t) for k, t in bd.search_level(left, R, grad, coarse, gp).items()}
+
+    def same(a, b, where):
+        for key in a:
+            if kw.get("fusion") and key == "energies":
+                continue  # not written
+            x, y = a[key][where], b[key][where]
+            assert np.array_equal(x, y, equal_nan=x.dtype.kind == "f"), key
+
+    a, b = run(L, G, near), run(L, G, far)
+    everywhere = np.ones(a["u_init"].shape, bool)
+    for coarse, ref in ((near, a), (far, b), (None, run(L, G, None))):
+        same(ref, run(odd(L), odd(G), coarse), everywhere)
+    same(a, b, a["u_init"] == b["u_init"])

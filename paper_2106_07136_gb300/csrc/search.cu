@@ -465,8 +465,10 @@ __device__ __forceinline__ void search_first_step(const SearchArgs &a, const Row
   float t;
   split_disp(st.D, kd, t);
   const int ib = xl + kd;
-  // a warp whose patches all sample inside [0, w - 2] masks and clamps nothing
-  if (kInnerPath<PS> && __all_sync(kFull, (unsigned)(kd + x0) <= (unsigned)(a.w - 1 - PS))) {
+  // a warp whose patches all sample inside [0, w - 2] masks and clamps nothing:
+  // kd + x0 in [0, w - 1 - PS], which no base is where the level is a patch wide
+  // (w >= PS: the right side is not negative)
+  if (kInnerPath<PS> && __all_sync(kFull, (unsigned)(kd + x0) < (unsigned)(a.w - PS))) {
     patch_sums<true>(a, st, act, full, PS, true, Lc, Gc);
     rows.ready();  // staged rows (if any) arrive while the sums above load
     patch_ab<true>(rows, st, ib, kd);

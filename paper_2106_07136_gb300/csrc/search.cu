@@ -489,8 +489,8 @@ __device__ __forceinline__ void search_first_step(const SearchArgs &a, const Row
 //     integer base. A patch whose base and gradient did not change gets the
 //     same sums again, so its result does not depend on its neighbours.
 // The valid set can only change near the image border: while every column of
-// the patch samples inside [0, w - 2] (kd in [-x0, w - 1 - PS - x0]) it is the
-// full set, with no per-column tests.
+// the patch samples inside [0, w - 2] (kd + x0 in [0, w - 1 - PS], no base at all
+// where the level is a patch wide) it is the full set, with no per-column tests.
 template <int PS, int CPL, bool SH, bool PAIR, class Rows>
 __device__ __forceinline__ bool search_next_step(const SearchArgs &a, const Rows &rows,
                                                  PatchState<PS, CPL, SH, PAIR> &st,
@@ -503,7 +503,7 @@ __device__ __forceinline__ bool search_next_step(const SearchArgs &a, const Rows
   const int kd = __float2int_rz(f);
   const int ib = (int)((unsigned)xl + (unsigned)kd);
   unsigned code = full;
-  if ((unsigned)kd + (unsigned)x0 > (unsigned)(a.w - 1 - PS)) code = valid_code<CPL>(act, ib, t, a.w);
+  if ((unsigned)kd + (unsigned)x0 >= (unsigned)(a.w - PS)) code = valid_code<CPL>(act, ib, t, a.w);
   const bool chg = !st.frozen && code != st.prev;
   const bool mv = !st.frozen && kd != st.kc;
   const unsigned r = __reduce_or_sync(kFull, (chg ? 1u : 0u) | (mv ? 2u : 0u) |

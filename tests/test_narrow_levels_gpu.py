@@ -1,11 +1,19 @@
 """Levels exactly a patch wide, and one column wider: every sample base but 0 (or 0 and 1) leaves
-columns outside the image, so the valid set of the first update follows the start."""
+columns outside the image, so the valid set follows the start and changes with the updates."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
+import torch
 
 import paper_2106_07136_gb300 as bd
+import synth
 from attribution import FLAG_DIVERGED
-from gpu_helpers import DROP, DSTAR_ATOL, decision_margins, dev, host, oracle_unstable
+from gpu_helpers import (DROP, DSTAR_ATOL, assert_explained, decision_margins, dev, host,
+                         oracle_unstable)
+from paper_2106_07136_gb300 import build as cuda_build
 
 pytestmark = pytest.mark.gpu
 
@@ -73,3 +81,93 @@ def check_against_oracle(orc, ps, wider, kw):
 def test_first_update_follows_the_start(orc, ps, wider, fusion):
     """One update from starts of a few pixels either way."""
     check_against_oracle(orc, ps, wider, dict(iterations=1, fusion=fusion))
+
+
+@pytest.mark.parametrize("ps", [8, 12, 16])
+@pytest.mark.parametrize("wider", [0, 1])
+@pytest.mark.parametrize("kw", [dict(fusion=0), dict(fusion=1), dict(normalize=0)])
+def test_later_updates_follow_the_base(orc, ps, wider, kw):
+    """The whole search: each base that an update reaches has its own valid set."""
+    check_against_oracle(orc, ps, wider, dict(iterations=12, **kw))
+
+
+def seeded_frames(w):
+    """Two frames of pairs whose coarsest level (of 4) is 8 columns at widths 113 to 128, and the
+    disparity of the frame before them."""
+    pairs = [synth.make_cfg2(seed=synth.stereo.pair_seed(6, i), h=160, w=w) for i in range(2)]
+    prev = np.stack([p.disp for p in pairs]).astype(np.float32)
+    return np.stack([p.left for p in pairs]), np.stack([p.right for p in pairs]), prev
+
+
+NARROW_KW = dict(patch_size=8, overlap=0.75, iterations=12, coarsest_scale=4, finest_scale=0,
+                 gamma=0.5)
+
+
+@pytest.mark.parametrize("w", [113, 128])
+def test_warm_start_on_a_coarsest_level_of_one_patch(orc, w):
+    L, R, prev = seeded_frames(w)
+    gp, op = bd.default_params(**NARROW_KW), orc.OracleParams.make(**NARROW_KW)
+    m = bd.Matcher()
+    out = host(m.match_warm(dev(L, torch.uint8), dev(R, torch.uint8), dev(prev), gp))
+    m.close()
+    for i in range(2):
+        assert_explained(orc, out[i], L[i], R[i], gp, op, f"{w} wide, frame {i}", budget=False,
+                         prev=prev[i])
+
+
+CHECKED = """
+import sys
+import numpy as np
+sys.path[:0] = sys.argv[2:]
+import paper_2106_07136_gb300 as bd
+import oracle
+import test_narrow_levels_gpu as t
+assert bd.checked_build()
+out = t.narrow_outputs(oracle)
+out["__sites__"] = np.array([bd.check_status()], dtype=np.int64)
+np.savez(sys.argv[1], **out)
+"""
+
+
+def narrow_outputs(orc):
+    out = {}
+    L, R, prev = seeded_frames(128)
+    gp = bd.default_params(**NARROW_KW)
+    m = bd.Matcher()
+    net = bd.ProposalNet(bd.net_init_weights(seed=5))
+    for variant, tiled in LAYOUTS:
+        bd.set_search_variant(variant)
+        bd.set_search_tiling(tiled)
+        key = f"{variant} {tiled}"
+        Ld, Rd = dev(L, torch.uint8), dev(R, torch.uint8)
+        out["warm " + key] = host(m.match_warm(Ld, Rd, dev(prev), gp))
+        out["learned " + key] = host(m.match_learned(net, Ld, Rd, gp, fallback=True))
+        for ps in (8, 12, 16):
+            for wider in (0, 1):
+                o, _ = narrow_level(orc, ps, ps + wider, 97, dict(iterations=12), 12.0, ps)
+                p = bd.default_params(patch_size=ps, overlap=0.75, gamma=0.25)
+                g = bd.search_level(dev(o["L"]), bd.pack_right(dev(o["R"])), dev(o["G"]),
+                                    dev(o["coarse"]), p)
+                out.update({f"{ps}+{wider} {k} {key}": host(v) for k, v in g.items()})
+    net.close()
+    m.close()
+    return out
+
+
+def test_checked_build_catches_nothing(orc, tmp_path):
+    """Starts up to 12 px either way: no access of the bounds-checked build is out of bounds, and
+    every output is the normal build's bit for bit."""
+    lib = cuda_build.build(checked=True)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    (tmp_path / "child.py").write_text(CHECKED)
+    res = tmp_path / "out.npz"
+    r = subprocess.run([sys.executable, str(tmp_path / "child.py"), str(res), root,
+                        os.path.join(root, "tests")], env=dict(os.environ, BDIS_LIBRARY=lib),
+                       cwd=root, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+    got = dict(np.load(res))
+    assert int(got.pop("__sites__")[0]) == 0
+    ref = narrow_outputs(orc)
+    assert set(got) == set(ref)
+    for k in ref:
+        assert np.array_equal(got[k], ref[k], equal_nan=ref[k].dtype.kind == "f"), k

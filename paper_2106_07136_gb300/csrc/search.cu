@@ -220,7 +220,11 @@ struct TileRows {
   __device__ __forceinline__ const float2 *col_clamped(int x) const {
     return tile + min(max(x - lo, 0), width - 1);
   }
-  __device__ __forceinline__ float2 ld(const float2 *p, int r) const { return p[r * TW]; }
+  __device__ __forceinline__ float2 ld(const float2 *p, int r) const {
+    BDIS_CHECKED_ONLY(if (!in_bounds(p - tile, width, kCheckSearchSample))
+                          return make_float2(0.f, 0.f);)
+    return p[r * TW];
+  }
   // the staging copies of this lane are complete and the warp's are visible
   __device__ __forceinline__ void ready() const {
     asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -750,7 +754,9 @@ __device__ __forceinline__ void fixed_patch(const SearchArgs &a, const Rows &row
   int kd;
   float t;
   split_disp(D, kd, t);
-  const int ib = xl + kd;
+  // (where a group has lanes past its patch, they read its first columns, unused:
+  // their own may lie outside a staged tile)
+  const int ib = (PS == CPL * G || act[0] ? xl : x0) + kd;
   // samples at D* + {-1, 0, 1} have fraction t; at D* +- 0.5 fraction th, with
   // base column one further right when t >= 0.5
   const bool hi = t >= 0.5f;

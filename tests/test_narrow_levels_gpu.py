@@ -154,20 +154,88 @@ def narrow_outputs(orc):
     return out
 
 
-def test_checked_build_catches_nothing(orc, tmp_path):
-    """Starts up to 12 px either way: no access of the bounds-checked build is out of bounds, and
-    every output is the normal build's bit for bit."""
+def checked_outputs(script, tmp_path):
+    """The arrays that `script` saves in a process that loads the bounds-checked build."""
     lib = cuda_build.build(checked=True)
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    (tmp_path / "child.py").write_text(CHECKED)
+    (tmp_path / "child.py").write_text(script)
     res = tmp_path / "out.npz"
     r = subprocess.run([sys.executable, str(tmp_path / "child.py"), str(res), root,
                         os.path.join(root, "tests")], env=dict(os.environ, BDIS_LIBRARY=lib),
                        cwd=root, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
-    got = dict(np.load(res))
+    return dict(np.load(res))
+
+
+def test_checked_build_catches_nothing(orc, tmp_path):
+    """Starts up to 12 px either way: no access of the bounds-checked build is out of bounds, and
+    every output is the normal build's bit for bit."""
+    got = checked_outputs(CHECKED, tmp_path)
     assert int(got.pop("__sites__")[0]) == 0
     ref = narrow_outputs(orc)
     assert set(got) == set(ref)
     for k in ref:
         assert np.array_equal(got[k], ref[k], equal_nan=ref[k].dtype.kind == "f"), k
+
+
+TILE = """
+import sys
+import numpy as np
+sys.path[:0] = sys.argv[2:]
+import paper_2106_07136_gb300 as bd
+import test_narrow_levels_gpu as t
+assert bd.checked_build()
+out = t.full_tile_outputs()
+out["__sites__"] = np.array([bd.check_status()], dtype=np.int64)
+np.savez(sys.argv[1], **out)
+"""
+
+
+def full_tile_level(span):
+    """Patches of 12 columns, 6 apart, one row of them: two neighbours that share a warp of the
+    one-column-per-lane layout start `span` px apart, so that the columns their ranges reach are
+    47 + span, and each takes one step of -11.5 px, nearly its whole range, inside the image."""
+    ps, w, first, start = 12, 204, 12, -30.0  # patch indices first and first + 1
+    x = np.arange(w, dtype=np.float64)
+    L = np.broadcast_to(2 * x, (ps, w))
+    G = np.full((ps, w), 2.0)
+    mid = 6 * first - start + 12 + span / 2  # between the two patches' samples
+    R = np.where(x < mid, 2 * (x + start) - 23, 2 * (x + start - span) - 23)
+    coarse = np.zeros((ps // 2, w // 2))
+    for i, u in ((first, start), (first + 1, start - span)):
+        coarse[:, 3 * i + 2:3 * i + 4] = u / 2  # patch i's centre is at 3 i + 2.75
+    kw = dict(patch_size=ps, overlap=0.5, iterations=1, normalize=0, gamma=0.25)
+    return L, np.broadcast_to(R, (ps, w)), G, coarse, kw, first
+
+
+SPANS = [46, 47, 48, 49]  # 48 fills the tile's 96 columns; 49 is read from global memory
+
+
+def full_tile_outputs():
+    out = {}
+    for span in SPANS:
+        L, R, G, coarse, kw, _ = full_tile_level(span)
+        for tiled in (False, True):
+            bd.set_search_variant(1)
+            bd.set_search_tiling(tiled)
+            g = bd.search_level(dev(L), bd.pack_right(dev(R)), dev(G), dev(coarse),
+                                bd.default_params(**kw))
+            out.update({f"{span} {tiled} {k}": host(v) for k, v in g.items()})
+    return out
+
+
+def test_lanes_past_the_patch_stay_in_a_full_tile(tmp_path):
+    """Patch 12, one column per lane: four lanes of each group have no column. On a tile whose
+    columns are all used, the bounds-checked build finds no read past it; outputs as untiled."""
+    got = checked_outputs(TILE, tmp_path)
+    assert int(got.pop("__sites__")[0]) == 0
+    ref = full_tile_outputs()
+    for span in SPANS:
+        first = full_tile_level(span)[-1]
+        d, u = ref[f"{span} True d_star"][0, 0], ref[f"{span} True u_init"][0, 0]
+        np.testing.assert_allclose((d - u)[first:first + 2], -11.5, atol=1e-3)
+        np.testing.assert_allclose(u[first] - u[first + 1], span, atol=1e-3)
+    for k in ref:
+        assert np.array_equal(got[k], ref[k], equal_nan=ref[k].dtype.kind == "f"), k
+        assert np.array_equal(ref[k], ref[k.replace("True", "False")],
+                              equal_nan=ref[k].dtype.kind == "f"), k

@@ -1265,12 +1265,14 @@ struct bdis_net {
   int part_blocks = 0;
   // device word set when a forward kernel's bounded wait ran out
   int *fault = nullptr;
-  unsigned *sync = nullptr;  // grid barrier counter of the fused inference kernel
   // activations in the padded planar layout for count h x w images: of
   // inference, and of training (with the gradients of the layers' outputs)
   struct Planar {
     __nv_bfloat16 *x0 = nullptr, *a[5] = {}, *g[5] = {}, *g6 = nullptr;
     float *map = nullptr;  // training: the forward map
+    // grid barrier counter of the launches on these buffers (its own, so that a
+    // forward pass and a gradient on two streams share nothing they write)
+    unsigned *sync = nullptr;
     int h = 0, w = 0, count = 0;
     size_t plane_cap = 0, map_cap = 0;  // bytes allocated per plane, and of the map
   } infer, train;
@@ -1321,11 +1323,13 @@ bdis_status net_reserve_planar(bdis_net::Planar &p, int h, int w, int count, boo
   else
     net_free_planar(p);
   p.h = p.w = p.count = 0;
-  auto take = [&](__nv_bfloat16 *&q, int planes) {
-    if (e == cudaSuccess && !fits) e = bdis::device_alloc((void **)&q, planes * plane);
+  auto take = [&](__nv_bfloat16 *&q, int planes, size_t extra = 0) {
+    if (e == cudaSuccess && !fits) e = bdis::device_alloc((void **)&q, planes * plane + extra);
     if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, planes * plane, st);
   };
-  take(p.x0, 2);
+  take(p.x0, 2, sizeof(unsigned));  // the counter behind the planes
+  if (e == cudaSuccess && !fits)
+    p.sync = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(p.x0) + 2 * plane);
   for (auto &q : p.a) take(q, 4);
   if (train) {
     for (auto &q : p.g) take(q, 4);
@@ -1554,9 +1558,8 @@ bool launch_chain(bdis_net *n, BandNet &net, int H, int W, int count, cudaStream
   net.W = W;
   net.count = count;
   net.slab_bytes = slab;
-  net.sync = n->sync;
   net.fault = n->fault;
-  if (cudaMemsetAsync(n->sync, 0, sizeof(unsigned), st) != cudaSuccess) {
+  if (cudaMemsetAsync(net.sync, 0, sizeof(unsigned), st) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -1585,6 +1588,7 @@ bool forward_planar(bdis_net *n, const bdis_net::Planar &p, const float *L3, con
   net.L = L3;
   net.R = R3;
   net.r_stride = r_stride;
+  net.sync = p.sync;
   return launch_chain<false>(n, net, H, W, count, st);
 }
 
@@ -1604,6 +1608,7 @@ bool backward_planar(bdis_net *n, const bdis_net::Planar &p, const float *label,
   net.map = p.map;
   net.label = label;
   net.loss = n->loss;
+  net.sync = p.sync;
   if (cudaMemsetAsync(n->loss, 0, sizeof(float), st) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -1690,7 +1695,6 @@ void net_release(bdis_net *n) {
   cudaFree(n->grad);
   cudaFree(n->loss);
   cudaFree(n->fault);
-  cudaFree(n->sync);
   for (int l = 0; l < kLayers; ++l) {
     cudaFree(n->wf[l]);
     cudaFree(n->wb[l]);
@@ -1753,7 +1757,6 @@ bdis_status bdis_net_create(int device, const float *weights, bdis_net **out) {
   alloc((void **)&n->grad, wb);
   alloc((void **)&n->loss, sizeof(float));
   alloc((void **)&n->fault, sizeof(int));
-  alloc((void **)&n->sync, sizeof(unsigned));
   for (int l = 0; l < kLayers; ++l) {
     alloc((void **)&n->wf[l], 2 * kCoutP[l] * 9 * kCinP[l]);
     if (l > 0) alloc((void **)&n->wb[l], 2 * kCoutP[l] * 9 * kCinP[l]);

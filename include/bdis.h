@@ -542,19 +542,22 @@ bdis_status bdis_net_train_step(bdis_net *net, const float *L, const float *R, i
                                 int width, int height, int count, const float *label, float lr,
                                 float *loss_out, void *stream);
 
-/* Whether a forward pass of the network timed out since the last call:
- * waits for `stream`, then returns BDIS_E_TIMEOUT (and clears the record) if
- * a tensor-core forward kernel's bounded wait for its own MMAs (about 200 ms)
- * ran out since the last bdis_net_status; that kernel then wrote NaN for the
- * tile and returned, so a proposal (and bdis_match_learned's seed) may hold
- * NaN there, which the seed map treats as missing. BDIS_OK otherwise. The
- * forward entry points themselves return before the kernels run, so this is
- * how a caller learns of it. */
+/* Whether a call of the network timed out since the last bdis_net_status:
+ * waits for `stream`, then returns BDIS_E_TIMEOUT (and clears the record) if a
+ * bounded wait of one of its kernels ran out (about 200 ms for a kernel's own
+ * MMAs and copies, 1 s at a grid barrier), else BDIS_OK. A forward kernel then
+ * wrote NaN for its part of the proposal and returned, so a proposal (and
+ * bdis_match_learned's seed) may hold NaN there, which the seed map treats as
+ * missing. A gradient in any of whose kernels a wait ran out gives a loss and a
+ * gradient of NaN, and bdis_net_train_step then leaves the weights and Adam's
+ * moments as they are (the step counts for Adam's bias corrections). Entry points
+ * that return before their kernels run can report it in no other way. */
 bdis_status bdis_net_status(bdis_net *net, void *stream);
 
 /* Host-side fault injection, for tests of the path above: records a timeout
- * exactly as the kernel's timeout path does (the network's device fault word
- * is written from the host); the next bdis_net_status returns BDIS_E_TIMEOUT. */
+ * exactly as a kernel's timeout path does (the network's device fault word
+ * is written from the host); the next bdis_net_status returns BDIS_E_TIMEOUT, and
+ * a gradient or training step before it runs as one whose wait ran out. */
 bdis_status bdis_net_inject_timeout(bdis_net *net);
 
 /* Copy the FP32 master weights to host memory (waits for the device). */

@@ -544,12 +544,12 @@ class ProposalNet:
         return loss.value
 
     def status(self, stream=None):
-        """bdis_net_status: raise BdisError (BDIS_E_TIMEOUT) if a forward pass's
-        bounded wait ran out since the last check; waits for the stream."""
+        """bdis_net_status: raise BdisError (BDIS_E_TIMEOUT) if a bounded wait of a
+        forward pass or of a gradient ran out since the last check; waits for the stream."""
         check(self._lib.bdis_net_status(self._h, _stream_ptr(stream)), "bdis_net_status")
 
     def inject_timeout(self):
-        """Host-side fault injection: record a forward-pass timeout."""
+        """Host-side fault injection: record a timeout, also for the next gradient."""
         check(self._lib.bdis_net_inject_timeout(self._h), "bdis_net_inject_timeout")
 
     def weights(self) -> np.ndarray:

@@ -443,7 +443,9 @@ __global__ void __launch_bounds__(128) conv_tc_kernel(
 // word, waits (bounded) for its own copies and MMAs in flight, writes NaN
 // over its bands of the map, frees its tensor memory and returns; the other
 // blocks then time out at the next grid barrier, if there is one, and do
-// the same.
+// the same. In training the word is the call's own, which its last kernel reads:
+// a call with a failed wait in any of its kernels gives a loss and a gradient of
+// NaN, and takes no Adam step.
 constexpr int kPad = 4;                // frame border = the largest dilation
 constexpr int kBandCols = 256;         // tensor-memory columns per accumulator (two)
 constexpr int kBandSmem = 224 * 1024;  // dynamic shared memory per block (one per SM)
@@ -846,13 +848,10 @@ __global__ void __launch_bounds__(kBandThreads, 1) net_chain_kernel(const BandNe
     if (ok) ok = band_layer<32, 16, kFwdLinearF32>(net, net.layer[5], sh, sbias, kg);
   }
   if (!ok) {
-    // a wait ran out (ok is uniform over the block): record it, and mark the
-    // loss, or this block's bands of the map, as missing (NaN), whatever was
-    // written there
+    // a wait ran out (ok is uniform over the block): record it, and mark this
+    // block's bands of the map as missing (NaN), whatever was written there
     if (tid == 0) atomicOr(net.fault, 1);
-    if constexpr (BACK) {
-      if (tid == 0) atomicExch(net.loss, __int_as_float(0x7fc00000));
-    } else {
+    if constexpr (!BACK) {
       const BandLayer &ly = net.layer[5];
       const int H = net.H, W = net.W, nb = (H + ly.BH - 1) / ly.BH;
       const long long units = (long long)net.count * nb;
@@ -1133,10 +1132,7 @@ __global__ void __launch_bounds__(128, kWgPerSm) conv_wgrad_kernel(const WgradAr
     ok = wgrad_layer<PLANAR, 32, 4, 16, 1>(args, args.layer[5], wg_smem, mbar, part);
   else
     ok = wgrad_layer<PLANAR, 32, 4, 32, 4>(args, args.layer[l], wg_smem, mbar, part);
-  if (!ok) {  // reported by bdis_net_status; the gradient is not a number
-    if (threadIdx.x == 0) atomicOr(args.fault, 1);
-    for (int i = threadIdx.x; i < kPart; i += 128) part[i] = __int_as_float(0x7fc00000);
-  }
+  if (!ok && threadIdx.x == 0) atomicOr(args.fault, 1);  // the sum below is then not a number
 }
 
 struct LayerBlocks {
@@ -1158,10 +1154,16 @@ __device__ __forceinline__ MasterAt master_at(int i) {
 }
 
 // The blocks' partial sums in master order: a block takes 32 elements, warp s
-// the partials s, s + 8, ..., and the eight sums are added in order.
+// the partials s, s + 8, ..., and the eight sums are added in order. Where a wait
+// of the call's kernels ran out (`failed`), what they left is partly that of an
+// earlier call: the loss and the gradient become NaN, and the network's fault
+// word is set, for bdis_net_status.
 __global__ void __launch_bounds__(256) reduce_grad_kernel(const float *__restrict__ part,
                                                           const LayerBlocks lb,
-                                                          float *__restrict__ grad) {
+                                                          float *__restrict__ grad,
+                                                          const int *__restrict__ failed,
+                                                          float *__restrict__ loss,
+                                                          int *__restrict__ fault) {
   __shared__ float slice[8][32];
   bdis::pdl_enter();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
@@ -1178,7 +1180,12 @@ __global__ void __launch_bounds__(256) reduce_grad_kernel(const float *__restric
   __syncthreads();
   if (warp == 0 && i < kMasterCount) {
     for (int s = 1; s < 8; ++s) sum += slice[s][lane];
-    grad[i] = sum;
+    const bool bad = __ldcg(failed) != 0;
+    grad[i] = bad ? __int_as_float(0x7fc00000) : sum;
+    if (bad && i == 0) {
+      *loss = __int_as_float(0x7fc00000);
+      atomicOr(fault, 1);
+    }
   }
 }
 
@@ -1223,12 +1230,12 @@ __global__ void bias_pad_kernel(const float *__restrict__ master, float *bias, i
   if (c < coutP) bias[c] = c < cout ? master[off + c] : 0.f;
 }
 
-// Adam on the master weights.
+// Adam on the master weights; none of it where the gradient's call failed.
 __global__ void adam_kernel(float *__restrict__ w, float *__restrict__ m, float *__restrict__ v,
                             const float *__restrict__ grad, int n, float lr, float b1, float b2,
-                            float eps, float c1, float c2) {
+                            float eps, float c1, float c2, const int *__restrict__ failed) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || __ldcg(failed) != 0) return;
   const float gr = grad[i];
   const float mi = b1 * m[i] + (1.f - b1) * gr;
   const float vi = b2 * v[i] + (1.f - b2) * gr * gr;
@@ -1254,7 +1261,11 @@ struct bdis_net {
   // per-layer padded bf16 weights, transposed copies, padded biases
   __nv_bfloat16 *wf[kLayers] = {}, *wb[kLayers] = {};
   float *bias[kLayers] = {};
+  // the loss, and the word that a wait of a gradient's kernels sets when it runs
+  // out; both cleared when a gradient begins
   float *loss = nullptr;
+  int *failed = nullptr;
+  bool inject = false;  // the next gradient begins as failed (for tests)
   long long step = 0;
   // activations for `cap` pixels
   long long cap = 0;
@@ -1263,7 +1274,8 @@ struct bdis_net {
   float *z6 = nullptr;
   float *part = nullptr;  // partial weight gradients, one per block of conv_wgrad_kernel
   int part_blocks = 0;
-  // device word set when a forward kernel's bounded wait ran out
+  // device word for bdis_net_status: a bounded wait of a forward pass or of a
+  // gradient's kernels ran out
   int *fault = nullptr;
   // activations in the padded planar layout for count h x w images: of
   // inference, and of training (with the gradients of the layers' outputs)
@@ -1558,7 +1570,6 @@ bool launch_chain(bdis_net *n, BandNet &net, int H, int W, int count, cudaStream
   net.W = W;
   net.count = count;
   net.slab_bytes = slab;
-  net.fault = n->fault;
   if (cudaMemsetAsync(net.sync, 0, sizeof(unsigned), st) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -1574,9 +1585,11 @@ bool launch_chain(bdis_net *n, BandNet &net, int H, int W, int count, cudaStream
 }
 
 // The forward pass as one cooperative launch: level planes in, the proposal
-// (channel 0 of the last layer) written straight to `out`.
+// (channel 0 of the last layer) written straight to `out`. `fault`: the word that
+// a wait which ran out sets.
 bool forward_planar(bdis_net *n, const bdis_net::Planar &p, const float *L3, const float *R3,
-                    int r_stride, int H, int W, int count, float *out, cudaStream_t st) {
+                    int r_stride, int H, int W, int count, float *out, int *fault,
+                    cudaStream_t st) {
   BandNet net{};
   for (int l = 0; l < 6; ++l) {
     net.layer[l].in = l ? p.a[l - 1] : p.x0;
@@ -1589,6 +1602,7 @@ bool forward_planar(bdis_net *n, const bdis_net::Planar &p, const float *L3, con
   net.R = R3;
   net.r_stride = r_stride;
   net.sync = p.sync;
+  net.fault = fault;
   return launch_chain<false>(n, net, H, W, count, st);
 }
 
@@ -1609,23 +1623,20 @@ bool backward_planar(bdis_net *n, const bdis_net::Planar &p, const float *label,
   net.label = label;
   net.loss = n->loss;
   net.sync = p.sync;
-  if (cudaMemsetAsync(n->loss, 0, sizeof(float), st) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
+  net.fault = n->failed;
   return launch_chain<true>(n, net, H, W, count, st);
 }
 
 cudaError_t forward(bdis_net *n, const float *L3, const float *R3, int r_stride, int H, int W,
-                    long long total, cudaStream_t st) {
+                    long long total, int *fault, cudaStream_t st) {
   pack_input_kernel<<<nblocks(total, 256), 256, 0, st>>>(L3, R3, r_stride, total, n->x0);
   conv<16, 32, kFwdRelu>(n->x0, n->wf[0], n->bias[0], kDil[0], H, W, total, nullptr, n->a[0],
-                         n->fault, st);
+                         fault, st);
   for (int l = 1; l < 5; ++l)
     conv<32, 32, kFwdRelu>(n->a[l - 1], n->wf[l], n->bias[l], kDil[l], H, W, total, nullptr,
-                           n->a[l], n->fault, st);
+                           n->a[l], fault, st);
   conv<32, 16, kFwdLinearF32>(n->a[4], n->wf[5], n->bias[5], kDil[5], H, W, total, nullptr,
-                              n->z6, n->fault, st);
+                              n->z6, fault, st);
   return cudaGetLastError();
 }
 
@@ -1660,7 +1671,7 @@ cudaError_t weight_gradients(bdis_net *n, const bdis_net::Planar *p, int H, int 
   wa.W = W;
   wa.count = count;
   wa.part = n->part;
-  wa.fault = n->fault;
+  wa.fault = n->failed;
   auto kernel = p ? conv_wgrad_kernel<true> : conv_wgrad_kernel<false>;
   cudaError_t e =
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
@@ -1669,7 +1680,15 @@ cudaError_t weight_gradients(bdis_net *n, const bdis_net::Planar *p, int H, int 
                                       st, wa);
   if (e == cudaSuccess)
     e = bdis::launch_maybe_overlapped(reduce_grad_kernel, dim3(nblocks(kMasterCount, 32)),
-                                      dim3(256), 0, st, (const float *)n->part, lb, n->grad);
+                                      dim3(256), 0, st, (const float *)n->part, lb, n->grad,
+                                      (const int *)n->failed, n->loss, n->fault);
+  return e;
+}
+
+// Begins a gradient: its loss and its word for failed waits.
+cudaError_t begin_gradient(bdis_net *n, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(n->loss, 0, sizeof(float) + sizeof(int), st);
+  if (e == cudaSuccess && n->inject) e = cudaMemsetAsync(n->failed, 1, sizeof(int), st);
   return e;
 }
 
@@ -1677,10 +1696,10 @@ cudaError_t weight_gradients(bdis_net *n, const bdis_net::Planar *p, int H, int 
 void data_gradients(bdis_net *n, int H, int W, long long total, cudaStream_t st) {
   // g5 = (W6^T g6) * relu'(a5)
   conv<16, 32, kBwdDataMasked>(n->g6, n->wb[5], nullptr, kDil[5], H, W, total, n->a[4],
-                               n->gact[4], n->fault, st);
+                               n->gact[4], n->failed, st);
   for (int l = 4; l >= 1; --l)
     conv<32, 32, kBwdDataMasked>(n->gact[l], n->wb[l], nullptr, kDil[l], H, W, total,
-                                 n->a[l - 1], n->gact[l - 1], n->fault, st);
+                                 n->a[l - 1], n->gact[l - 1], n->failed, st);
 }
 
 void net_release(bdis_net *n) {
@@ -1714,12 +1733,12 @@ bdis_status net_forward_on(bdis_net *n, const float *L, const float *R, int r_st
   if (g_net_tc == 1 && band_fits(h, w)) {
     bdis_status s = net_reserve_planar(n->infer, h, w, count, false, st);
     if (s != BDIS_OK) return s;
-    if (forward_planar(n, n->infer, L, R, r_stride, h, w, count, out, st))
+    if (forward_planar(n, n->infer, L, R, r_stride, h, w, count, out, n->fault, st))
       return record_cuda(cudaGetLastError());
   }
   bdis_status s = net_reserve(n, total, false);
   if (s != BDIS_OK) return s;
-  cudaError_t e = forward(n, L, R, r_stride, h, w, total, st);
+  cudaError_t e = forward(n, L, R, r_stride, h, w, total, n->fault, st);
   if (e == cudaSuccess) {
     take_channel0_kernel<<<nblocks(total, 256), 256, 0, st>>>(n->z6, total, out);
     e = cudaGetLastError();
@@ -1755,7 +1774,8 @@ bdis_status bdis_net_create(int device, const float *weights, bdis_net **out) {
   alloc((void **)&n->m, wb);
   alloc((void **)&n->v, wb);
   alloc((void **)&n->grad, wb);
-  alloc((void **)&n->loss, sizeof(float));
+  alloc((void **)&n->loss, sizeof(float) + sizeof(int));
+  n->failed = reinterpret_cast<int *>(n->loss + 1);
   alloc((void **)&n->fault, sizeof(int));
   for (int l = 0; l < kLayers; ++l) {
     alloc((void **)&n->wf[l], 2 * kCoutP[l] * 9 * kCinP[l]);
@@ -1810,16 +1830,17 @@ bdis_status bdis_net_gradient(bdis_net *n, const float *L3, const float *R3, int
     bdis_net::Planar &p = n->train;
     s = net_reserve_planar(p, height, width, count, true, st);
     if (s != BDIS_OK && s != BDIS_E_NOMEM) return s;
-    done = s == BDIS_OK &&
-           forward_planar(n, p, L3, R3, r_stride, height, width, count, p.map, st) &&
+    done = s == BDIS_OK && begin_gradient(n, st) == cudaSuccess &&
+           forward_planar(n, p, L3, R3, r_stride, height, width, count, p.map, n->failed, st) &&
            backward_planar(n, p, label, height, width, count, st);
     if (done) e = weight_gradients(n, &p, height, width, count, st);
   }
   if (!done) {
     s = net_reserve(n, total, true);
     if (s != BDIS_OK) return s;
-    e = forward(n, L3, R3, r_stride, height, width, total, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(n->loss, 0, sizeof(float), st);
+    e = begin_gradient(n, st);
+    if (e == cudaSuccess)
+      e = forward(n, L3, R3, r_stride, height, width, total, n->failed, st);
     if (e == cudaSuccess) {
       loss_kernel<<<nblocks(total, 256), 256, 0, st>>>(n->z6, label, total, 1.f / (float)total,
                                                        n->g6, n->loss);
@@ -1830,6 +1851,7 @@ bdis_status bdis_net_gradient(bdis_net *n, const float *L3, const float *R3, int
       e = weight_gradients(n, nullptr, height, width, count, st);
     }
   }
+  n->inject = false;
   if (e == cudaSuccess && loss_out)
     e = cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && grad_out)
@@ -1850,7 +1872,7 @@ bdis_status bdis_net_train_step(bdis_net *n, const float *L3, const float *R3, i
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)n->step), c2 = 1.f - powf(b2, (float)n->step);
   adam_kernel<<<nblocks(kMasterCount, 256), 256, 0, st>>>(n->w, n->m, n->v, n->grad, kMasterCount,
-                                                          lr, b1, b2, 1e-8f, c1, c2);
+                                                          lr, b1, b2, 1e-8f, c1, c2, n->failed);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = pack_all(n, st);
   if (e == cudaSuccess && loss_out) {
@@ -1878,10 +1900,11 @@ bdis_status bdis_net_status(bdis_net *n, void *stream) {
   int fault = 0;
   if (e == cudaSuccess) e = cudaMemcpy(&fault, n->fault, sizeof(int), cudaMemcpyDeviceToHost);
   if (e == cudaSuccess && fault) e = cudaMemset(n->fault, 0, sizeof(int));
+  n->inject = false;
   if (e != cudaSuccess) return bdis::record_cuda(e);
   if (fault) {
-    bdis::set_last_error("proposal network: a forward pass's bounded wait ran out (its tile "
-                         "was written as NaN)");
+    bdis::set_last_error("proposal network: a bounded wait of a forward pass (its tile was "
+                         "written as NaN) or of a gradient (its loss and gradient are NaN) ran out");
     return BDIS_E_TIMEOUT;
   }
   return BDIS_OK;
@@ -1892,6 +1915,7 @@ bdis_status bdis_net_inject_timeout(bdis_net *n) {
   const int one = 1;
   cudaError_t e = cudaSetDevice(n->device);
   if (e == cudaSuccess) e = cudaMemcpy(n->fault, &one, sizeof(int), cudaMemcpyHostToDevice);
+  n->inject = true;
   return bdis::record_cuda(e);
 }
 

@@ -7,6 +7,7 @@ import torch
 
 import paper_2106_07136_gb300 as bd
 from gpu_helpers import dev
+from paper_2106_07136_gb300 import _lib
 
 pytestmark = pytest.mark.gpu
 
@@ -44,4 +45,44 @@ def test_forward_beside_gradient(shape):
     assert len(grads) == 40 and passes > 0 and wrong == 0
     for loss, g in grads:
         assert np.array_equal(g, ref_g) and abs(loss - ref_loss) <= 1e-5 * abs(ref_loss)
+    net.close()
+
+
+@pytest.fixture
+def net_variant(request):
+    old = bd.get_net_variant()
+    bd.set_net_variant(request.param)
+    yield request.param
+    bd.set_net_variant(old)
+
+
+@pytest.mark.parametrize("net_variant", [0, 1, 2], indirect=True)
+def test_a_gradient_whose_wait_ran_out_is_not_a_number(net_variant):
+    """The call's word for failed waits, set from the host where a kernel would set it: loss and
+    gradient are NaN, a training step leaves the weights, the next calls are as always."""
+    L, R, label = net_batch(2, 3, 30, 40)
+    net = bd.ProposalNet(bd.net_init_weights(seed=6))
+    w0 = net.weights()
+    ref_loss, ref = net.gradient(L, R, label)
+
+    def reported():
+        with pytest.raises(bd.BdisError) as e:
+            net.status()
+        assert e.value.status == _lib.BDIS_E_TIMEOUT
+        net.status()
+
+    net.inject_timeout()
+    loss, g = net.gradient(L, R, label)
+    assert np.isnan(loss) and np.isnan(g).all()
+    reported()
+    net.inject_timeout()
+    assert np.isnan(net.train_step(L, R, label, 1e-3))
+    reported()
+    assert np.array_equal(net.weights(), w0)
+    loss, g = net.gradient(L, R, label)
+    assert np.array_equal(g, ref) and abs(loss - ref_loss) <= 1e-5 * abs(ref_loss)
+    assert abs(net.train_step(L, R, label, 1e-3) - ref_loss) <= 1e-5 * abs(ref_loss)
+    w1 = net.weights()
+    assert np.isfinite(w1).all() and not np.array_equal(w1, w0)
+    net.status()
     net.close()

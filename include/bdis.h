@@ -526,7 +526,12 @@ bdis_status bdis_net_create(int device, const float *weights, bdis_net **out);
 
 /* Proposal for count x h x w level planes: L (float), R (float with element
  * stride r_stride: 1 plain, 2 packed) -> disparity (float, level pixels).
- * All device. Activations are held by the network object (grown on demand). */
+ * All device. Activations are held by the network object (grown on demand; a
+ * call whose shape differs from the last one's waits for the device). Under
+ * stream capture, call it once with the same shape before: nothing can be
+ * allocated there. What a captured call uses then stays as it is while other
+ * shapes run, except for images that the default kernels do not take (below):
+ * there a larger batch gives the buffers back, and the graph with them. */
 bdis_status bdis_net_forward(bdis_net *net, const float *L, const float *R, int r_stride,
                              int width, int height, int count, float *disparity, void *stream);
 

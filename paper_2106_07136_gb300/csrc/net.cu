@@ -1287,7 +1287,12 @@ struct bdis_net {
     unsigned *sync = nullptr;
     int h = 0, w = 0, count = 0;
     size_t plane_cap = 0, map_cap = 0;  // bytes allocated per plane, and of the map
+    bool captured = false;  // a captured graph refers to them
+    bool holds(int hh, int ww, int cc) const { return h == hh && w == ww && count == cc; }
   } infer, train;
+  // those a captured graph refers to (and at most one more each) while other
+  // shapes run
+  std::vector<Planar> kept_infer, kept_train;
 };
 
 namespace {
@@ -1321,10 +1326,36 @@ void net_free_planar(bdis_net::Planar &p) {
 // device has finished with the one before: a
 // gradient of 64 and of 48 images of 40x30 in turn takes 247 us where reallocating
 // took 1115, a forward pass 78 where it took 535. Under capture nothing may be
-// waited for, and the buffers are allocated anew.
-bdis_status net_reserve_planar(bdis_net::Planar &p, int h, int w, int count, bool train,
-                               cudaStream_t st) {
-  if (p.h == h && p.w == w && p.count == count) return BDIS_OK;
+// waited for, and the buffers are allocated anew. Buffers that a captured graph
+// refers to serve their shape only (its launches rely on the borders) and go
+// aside, to `kept`, while another shape runs.
+bdis_status net_reserve_planar(bdis_net::Planar &p, std::vector<bdis_net::Planar> &kept, int h,
+                               int w, int count, bool train, cudaStream_t st) {
+  auto mark = [&]() {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (!p.captured && cudaStreamIsCapturing(st, &cap) == cudaSuccess &&
+        cap != cudaStreamCaptureStatusNone)
+      p.captured = true;
+  };
+  if (!p.holds(h, w, count))
+    for (auto &q : kept)
+      if (q.holds(h, w, count)) {
+        std::swap(p, q);
+        break;
+      }
+  if (p.holds(h, w, count)) {
+    mark();
+    return BDIS_OK;
+  }
+  if (p.captured) {
+    auto q = std::find_if(kept.begin(), kept.end(), [](auto &k) { return !k.captured; });
+    if (q != kept.end()) {
+      std::swap(p, *q);
+    } else {
+      kept.push_back(p);
+      p = bdis_net::Planar();
+    }
+  }
   const size_t plane = (size_t)pp_plane(h, w, count) * sizeof(__nv_bfloat16);
   const size_t map = train ? sizeof(float) * (size_t)h * w * count : 0;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1360,6 +1391,7 @@ bdis_status net_reserve_planar(bdis_net::Planar &p, int h, int w, int count, boo
   p.h = h;
   p.w = w;
   p.count = count;
+  mark();
   return BDIS_OK;
 }
 
@@ -1707,6 +1739,8 @@ void net_release(bdis_net *n) {
   net_free_acts(n);
   net_free_planar(n->infer);
   net_free_planar(n->train);
+  for (auto &p : n->kept_infer) net_free_planar(p);
+  for (auto &p : n->kept_train) net_free_planar(p);
   cudaFree(n->part);
   cudaFree(n->w);
   cudaFree(n->m);
@@ -1731,7 +1765,7 @@ bdis_status net_forward_on(bdis_net *n, const float *L, const float *R, int r_st
   const long long total = (long long)w * h * count;
   if (!g_sms) init_sms();
   if (g_net_tc == 1 && band_fits(h, w)) {
-    bdis_status s = net_reserve_planar(n->infer, h, w, count, false, st);
+    bdis_status s = net_reserve_planar(n->infer, n->kept_infer, h, w, count, false, st);
     if (s != BDIS_OK) return s;
     if (forward_planar(n, n->infer, L, R, r_stride, h, w, count, out, n->fault, st))
       return record_cuda(cudaGetLastError());
@@ -1828,7 +1862,7 @@ bdis_status bdis_net_gradient(bdis_net *n, const float *L3, const float *R3, int
   const double planar_bytes = 704.0 * (height + 2 * kPad) * (width + 2 * kPad) * (double)count;
   if (g_net_tc == 1 && planar_bytes <= 32e9 && band_fits(height, width)) {
     bdis_net::Planar &p = n->train;
-    s = net_reserve_planar(p, height, width, count, true, st);
+    s = net_reserve_planar(p, n->kept_train, height, width, count, true, st);
     if (s != BDIS_OK && s != BDIS_E_NOMEM) return s;
     done = s == BDIS_OK && begin_gradient(n, st) == cudaSuccess &&
            forward_planar(n, p, L3, R3, r_stride, height, width, count, p.map, n->failed, st) &&

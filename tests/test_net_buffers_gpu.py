@@ -86,3 +86,30 @@ def test_a_gradient_whose_wait_ran_out_is_not_a_number(net_variant):
     assert np.isfinite(w1).all() and not np.array_equal(w1, w0)
     net.status()
     net.close()
+
+
+@pytest.mark.parametrize("others", [[(2, 9, 12)], [(2, 9, 12), (8, 40, 50), (1, 61, 37), (2, 9, 12)]])
+def test_a_captured_forward_pass_outlives_other_shapes(others):
+    """Replays of a captured forward pass after eager calls of smaller and larger shapes (and the
+    captured one's) through the same network: the eager pass bit for bit."""
+    net = bd.ProposalNet(bd.net_init_weights(seed=6))
+    L, R, _ = net_batch(3, 4, 30, 40)
+    ref = net.forward(L, R)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        out = net.forward(L, R)
+    for i, shape in enumerate(others):
+        Lo, Ro, _ = net_batch(4 + i, *shape)
+        fresh = bd.ProposalNet(bd.net_init_weights(seed=6))
+        for _ in range(2):
+            o = net.forward(Lo, Ro)
+            assert torch.equal(o, fresh.forward(Lo, Ro))
+            out.zero_()
+            graph.replay()
+            assert torch.equal(out, ref)
+        fresh.close()
+        assert torch.equal(net.forward(L, R), ref)
+    torch.cuda.synchronize()
+    net.status()
+    net.close()

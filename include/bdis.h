@@ -537,7 +537,12 @@ bdis_status bdis_net_forward(bdis_net *net, const float *L, const float *R, int 
 
 /* Loss (Huber, delta 1, mean over all count*h*w pixels; NaN labels count 0)
  * and its gradient with respect to the master weights, without updating.
- * loss_out / grad_out: host pointers or NULL (then nothing is copied). */
+ * loss_out / grad_out: host pointers or NULL (then nothing is copied).
+ * The network keeps, beside what its forward passes use (352 B per position of
+ * images framed by 4 pixels on each side; 448 B per pixel of images that the
+ * default kernels do not take), 704 B per framed position; a batch past 32 GB of
+ * them, or for which they cannot be had, 768 B per pixel; 576 where those cannot
+ * be had. BDIS_E_NOMEM if these cannot either. */
 bdis_status bdis_net_gradient(bdis_net *net, const float *L, const float *R, int r_stride,
                               int width, int height, int count, const float *label,
                               float *loss_out, float *grad_out, void *stream);

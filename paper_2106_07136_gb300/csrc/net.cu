@@ -23,6 +23,7 @@
 // GEMM with rows = output channels, columns = (tap, input channel), K = pixels,
 // whose blocks write partial sums that a second kernel adds in a fixed order.
 #include <cuda_bf16.h>
+#include <limits.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -1269,8 +1270,10 @@ struct bdis_net {
   long long step = 0;
   // activations for `cap` pixels
   long long cap = 0;
-  // (gact[l]: gradient of layer l's output; the last layer's is g6)
+  // (gact: gradients of the layers' outputs, one each, or two for all layers in
+  // turn; the last layer's is g6)
   __nv_bfloat16 *x0 = nullptr, *a[5] = {}, *gact[5] = {}, *g6 = nullptr;
+  __nv_bfloat16 *gact_of(int l) const { return gact[2] ? gact[l] : gact[l & 1]; }
   float *z6 = nullptr;
   float *part = nullptr;  // partial weight gradients, one per block of conv_wgrad_kernel
   int part_blocks = 0;
@@ -1408,25 +1411,31 @@ bdis_status net_reserve_part(bdis_net *n) {
 }
 
 // NHWC activations for `pixels` pixels; with `train`, also the gradients of
-// every layer's output.
+// every layer's output (768 B per pixel in all). Where those cannot be had, two
+// gradient buffers that the layers take in turn (576 B), with the planar training
+// buffers given back.
 bdis_status net_reserve(bdis_net *n, long long pixels, bool train) {
   if (pixels <= n->cap && (!train || n->gact[0])) return BDIS_OK;
   pixels = std::max(pixels, n->cap);
-  net_free_acts(n);
-  cudaError_t e = cudaSuccess;
-  auto alloc = [&](void **p, size_t bytes) {
-    if (e == cudaSuccess) e = bdis::device_alloc(p, bytes);
-  };
-  alloc((void **)&n->x0, pixels * 16 * 2);
-  for (auto &p : n->a) alloc((void **)&p, pixels * 32 * 2);
-  if (train)
-    for (auto &p : n->gact) alloc((void **)&p, pixels * 32 * 2);
-  alloc((void **)&n->g6, pixels * 16 * 2);
-  alloc((void **)&n->z6, pixels * 16 * 4);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
+  cudaError_t e = cudaErrorMemoryAllocation;
+  for (int grads = train ? 5 : 0; e != cudaSuccess; grads = 2) {
     net_free_acts(n);
-    return BDIS_E_NOMEM;
+    e = cudaSuccess;
+    auto alloc = [&](void **p, size_t bytes) {
+      if (e == cudaSuccess) e = bdis::device_alloc(p, bytes);
+    };
+    alloc((void **)&n->x0, pixels * 16 * 2);
+    for (auto &p : n->a) alloc((void **)&p, pixels * 32 * 2);
+    for (int i = 0; i < grads; ++i) alloc((void **)&n->gact[i], pixels * 32 * 2);
+    alloc((void **)&n->g6, pixels * 16 * 2);
+    alloc((void **)&n->z6, pixels * 16 * 4);
+    if (e == cudaSuccess) break;
+    cudaGetLastError();
+    if (grads != 5) {
+      net_free_acts(n);
+      return BDIS_E_NOMEM;
+    }
+    if (!n->train.captured) net_free_planar(n->train);
   }
   n->cap = pixels;
   return BDIS_OK;
@@ -1672,16 +1681,14 @@ cudaError_t forward(bdis_net *n, const float *L3, const float *R3, int r_stride,
   return cudaGetLastError();
 }
 
-// Every layer's weight gradient in one launch, on planar activations or (p
-// null) NHWC ones, and the sum of its partials.
-cudaError_t weight_gradients(bdis_net *n, const bdis_net::Planar *p, int H, int W, int count,
-                             cudaStream_t st) {
+// The weight gradients' blocks and arguments, on planar activations or (p null)
+// NHWC ones.
+void plan_weight_gradients(bdis_net *n, const bdis_net::Planar *p, int H, int W, int count,
+                           WgradArgs &wa, LayerBlocks &lb) {
   // Blocks per layer: as many in all as run at once, in proportion to the
   // layers' work (a tile of the first or last layer is a fraction of a middle
   // one's)
   static const double kCost[kLayers] = {0.4, 1, 1, 1, 1, 0.6};
-  WgradArgs wa{};
-  LayerBlocks lb{};
   long long tiles[kLayers];
   double work = 0;
   for (int l = 0; l < kLayers; ++l) {
@@ -1696,7 +1703,7 @@ cudaError_t weight_gradients(bdis_net *n, const bdis_net::Planar *p, int H, int 
     lb.blocks[l] = (int)std::max(1ll, std::min(tiles[l], (long long)share));
     blocks += lb.blocks[l];
     wa.layer[l] = {p ? (l ? p->a[l - 1] : p->x0) : (l ? n->a[l - 1] : n->x0),
-                   p ? (l < 5 ? p->g[l] : p->g6) : (l < 5 ? n->gact[l] : n->g6), kDil[l],
+                   p ? (l < 5 ? p->g[l] : p->g6) : (l < 5 ? n->gact_of(l) : n->g6), kDil[l],
                    lb.first[l], lb.blocks[l]};
   }
   wa.H = H;
@@ -1704,17 +1711,31 @@ cudaError_t weight_gradients(bdis_net *n, const bdis_net::Planar *p, int H, int 
   wa.count = count;
   wa.part = n->part;
   wa.fault = n->failed;
-  auto kernel = p ? conv_wgrad_kernel<true> : conv_wgrad_kernel<false>;
+}
+
+// Every layer's weight gradient in one launch, or (only >= 0) that layer's.
+cudaError_t launch_weight_gradients(WgradArgs wa, const LayerBlocks &lb, bool planar, int only,
+                                    cudaStream_t st) {
+  int blocks = lb.first[kLayers - 1] + lb.blocks[kLayers - 1];
+  if (only >= 0) {  // the same blocks, numbered from 0
+    blocks = lb.blocks[only];
+    wa.part += (long long)lb.first[only] * kPart;
+    for (int l = 0; l < kLayers; ++l) wa.layer[l].first = l <= only ? 0 : INT_MAX;
+  }
+  auto kernel = planar ? conv_wgrad_kernel<true> : conv_wgrad_kernel<false>;
   cudaError_t e =
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
   if (e == cudaSuccess)
     e = bdis::launch_maybe_overlapped(kernel, dim3((unsigned)blocks), dim3(128), (size_t)kWgSmem,
                                       st, wa);
-  if (e == cudaSuccess)
-    e = bdis::launch_maybe_overlapped(reduce_grad_kernel, dim3(nblocks(kMasterCount, 32)),
-                                      dim3(256), 0, st, (const float *)n->part, lb, n->grad,
-                                      (const int *)n->failed, n->loss, n->fault);
   return e;
+}
+
+// The sum of the weight gradients' partials.
+cudaError_t sum_weight_gradients(bdis_net *n, const LayerBlocks &lb, cudaStream_t st) {
+  return bdis::launch_maybe_overlapped(reduce_grad_kernel, dim3(nblocks(kMasterCount, 32)),
+                                       dim3(256), 0, st, (const float *)n->part, lb, n->grad,
+                                       (const int *)n->failed, n->loss, n->fault);
 }
 
 // Begins a gradient: its loss and its word for failed waits.
@@ -1724,14 +1745,31 @@ cudaError_t begin_gradient(bdis_net *n, cudaStream_t st) {
   return e;
 }
 
-// The data gradients of NHWC activations, layer by layer.
-void data_gradients(bdis_net *n, int H, int W, long long total, cudaStream_t st) {
-  // g5 = (W6^T g6) * relu'(a5)
-  conv<16, 32, kBwdDataMasked>(n->g6, n->wb[5], nullptr, kDil[5], H, W, total, n->a[4],
-                               n->gact[4], n->failed, st);
-  for (int l = 4; l >= 1; --l)
-    conv<32, 32, kBwdDataMasked>(n->gact[l], n->wb[l], nullptr, kDil[l], H, W, total,
-                                 n->a[l - 1], n->gact[l - 1], n->failed, st);
+// The gradients of NHWC activations: the data gradients layer by layer, then all
+// weight gradients; each layer's weight gradient before its output's gradient is
+// overwritten, where two buffers hold those (the same blocks, so the same sums).
+cudaError_t gradients(bdis_net *n, int H, int W, int count, cudaStream_t st) {
+  const long long total = (long long)H * W * count;
+  const bool in_turn = !n->gact[2];
+  WgradArgs wa{};
+  LayerBlocks lb{};
+  plan_weight_gradients(n, nullptr, H, W, count, wa, lb);
+  cudaError_t e = cudaSuccess;
+  for (int l = 5; l >= 0 && e == cudaSuccess; --l) {
+    if (in_turn) e = launch_weight_gradients(wa, lb, false, l, st);
+    if (e != cudaSuccess || l == 0) break;
+    // g[l - 1] = (W^T g[l]) * relu'(a[l - 1])
+    if (l == 5)
+      conv<16, 32, kBwdDataMasked>(n->g6, n->wb[5], nullptr, kDil[5], H, W, total, n->a[4],
+                                   n->gact_of(4), n->failed, st);
+    else
+      conv<32, 32, kBwdDataMasked>(n->gact_of(l), n->wb[l], nullptr, kDil[l], H, W, total,
+                                   n->a[l - 1], n->gact_of(l - 1), n->failed, st);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess && !in_turn) e = launch_weight_gradients(wa, lb, false, -1, st);
+  if (e == cudaSuccess) e = sum_weight_gradients(n, lb, st);
+  return e;
 }
 
 void net_release(bdis_net *n) {
@@ -1856,8 +1894,8 @@ bdis_status bdis_net_gradient(bdis_net *n, const float *L3, const float *R3, int
   // the loss with the data gradients, and the weight gradients are one launch
   // each (64 images of 40x30: 310 us by per-layer launches, 228 now). Its
   // padded planes take 704 B per position where the NHWC ones take 768 B per
-  // pixel; a batch beyond 32 GB of them, or for which they cannot be had, keeps
-  // the NHWC form.
+  // pixel (576 at least); a batch beyond 32 GB of them, or for which they cannot be
+  // had, keeps the NHWC form.
   bool done = false;
   const double planar_bytes = 704.0 * (height + 2 * kPad) * (width + 2 * kPad) * (double)count;
   if (g_net_tc == 1 && planar_bytes <= 32e9 && band_fits(height, width)) {
@@ -1867,7 +1905,13 @@ bdis_status bdis_net_gradient(bdis_net *n, const float *L3, const float *R3, int
     done = s == BDIS_OK && begin_gradient(n, st) == cudaSuccess &&
            forward_planar(n, p, L3, R3, r_stride, height, width, count, p.map, n->failed, st) &&
            backward_planar(n, p, label, height, width, count, st);
-    if (done) e = weight_gradients(n, &p, height, width, count, st);
+    if (done) {
+      WgradArgs wa{};
+      LayerBlocks lb{};
+      plan_weight_gradients(n, &p, height, width, count, wa, lb);
+      e = launch_weight_gradients(wa, lb, true, -1, st);
+      if (e == cudaSuccess) e = sum_weight_gradients(n, lb, st);
+    }
   }
   if (!done) {
     s = net_reserve(n, total, true);
@@ -1880,10 +1924,7 @@ bdis_status bdis_net_gradient(bdis_net *n, const float *L3, const float *R3, int
                                                        n->g6, n->loss);
       e = cudaGetLastError();
     }
-    if (e == cudaSuccess) {
-      data_gradients(n, height, width, total, st);
-      e = weight_gradients(n, nullptr, height, width, count, st);
-    }
+    if (e == cudaSuccess) e = gradients(n, height, width, count, st);
   }
   n->inject = false;
   if (e == cudaSuccess && loss_out)

@@ -113,3 +113,31 @@ def test_a_captured_forward_pass_outlives_other_shapes(others):
     torch.cuda.synchronize()
     net.status()
     net.close()
+
+
+@pytest.mark.parametrize("net_variant", [0, 2], indirect=True)
+@pytest.mark.parametrize("shape", [(1, 2, 3), (3, 31, 41), (2, 9, 300)])
+def test_two_gradient_buffers_give_the_same_gradient(net_variant, shape):
+    """A batch whose layers' gradients cannot all be had holds two at a time: the gradient bit for
+    bit, on every call; where those cannot be had either, the failure is reported and the network
+    is usable."""
+    batch, tiny = net_batch(7, *shape), net_batch(8, 1, 1, 1)
+    ref_net, net = (bd.ProposalNet(bd.net_init_weights(seed=6)) for _ in range(2))
+    ref_loss, ref = ref_net.gradient(*batch)
+    net.gradient(*tiny)  # the sums' buffer, which does not depend on the shape
+    try:
+        bd.inject_alloc_failures(2)
+        with pytest.raises(bd.BdisError) as e:
+            net.gradient(*batch)
+        assert e.value.status == _lib.BDIS_E_NOMEM
+        bd.inject_alloc_failures(1)
+        got = [net.gradient(*batch) for _ in range(2)]
+    finally:
+        bd.inject_alloc_failures(0)
+    net.gradient(*tiny)
+    got.append(net.gradient(*batch))
+    for loss, g in got:
+        assert np.array_equal(g, ref) and abs(loss - ref_loss) <= 1e-5 * abs(ref_loss)
+    net.status()
+    net.close()
+    ref_net.close()

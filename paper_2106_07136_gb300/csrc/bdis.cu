@@ -900,8 +900,24 @@ namespace {
 // 575 -> 389 (two chunks 422), 16 pairs 783 -> 650 (one chunk 665), 32 pairs 1258
 // -> 1130 (one 1202, three 1142), 64 pairs 2072 -> 1953 (two 2075, four 2017), 128
 // pairs 3677 -> 3611, 512 pairs 13350 -> 13240 (three 13780). A middle chunk past
-// 32 GB of workspace keeps the even split, whose chunks are smaller.
+// 32 GB of workspace keeps the even split, whose chunks are smaller; so does a
+// batch whose workspace cannot be had.
 constexpr int kHostChunks = 5;
+
+// Chunks of at most a third of the batch (a quarter from 8 pairs): from 32 pairs
+// the first and last are a sixteenth of it, and three equal ones lie between.
+int even_chunks(int count, int (&n)[kHostChunks]) {
+  if (count >= 32) {
+    n[0] = n[4] = count / 16;
+    n[1] = n[2] = (count - 2 * n[0]) / 3;
+    n[3] = count - 2 * n[0] - 2 * n[1];
+    return 5;
+  }
+  const int per = count >= 8 ? (count + 3) / 4 : (count + 1) / 2;
+  int k = 0;
+  for (int left = count; left > 0; left -= per) n[k++] = std::min(per, left);
+  return k;
+}
 
 int host_chunks(int w, int h, int count, const bdis_params &p, int (&n)[kHostChunks]) {
   const double pairs = (double)w * h * count / (640.0 * 480.0);
@@ -927,12 +943,8 @@ int host_chunks(int w, int h, int count, const bdis_params &p, int (&n)[kHostChu
     k = 5;
   }
   const int largest = *std::max_element(n, n + k);
-  if (k > 1 && plan_layout(w, h, largest, p, true).bytes > (32ull << 30) && count >= 5) {
-    k = 5;
-    n[0] = n[4] = part(1.0 / 16);
-    n[1] = n[2] = (count - n[0] - n[4]) / 3;
-    n[3] = count - n[0] - n[4] - n[1] - n[2];
-  }
+  if (k > 1 && plan_layout(w, h, largest, p, true).bytes > (32ull << 30))
+    return even_chunks(count, n);
   return k;
 }
 
@@ -968,25 +980,34 @@ bdis_status bdis_match_host(bdis_handle *h, const uint8_t *left, const uint8_t *
   // (i & 1); a slot is refilled only after the match that read it (ev_done)
   // and the copy-out that read its output (ev_out) have finished.
   int chunk_first[kHostChunks], chunk_n[kHostChunks];
-  const int nchunk = host_chunks(width, height, count, *p, chunk_n);
-  int cs = 0;
-  for (int i = 0, f = 0; i < nchunk; ++i) {
-    chunk_first[i] = f;
-    f += chunk_n[i];
-    cs = std::max(cs, chunk_n[i]);
+  int nchunk = host_chunks(width, height, count, *p, chunk_n);
+  Layout lay;
+  size_t slot_l[2], slot_r[2], slot_o[2];
+  for (bool even = false;; even = true) {
+    int cs = 0;
+    for (int i = 0, f = 0; i < nchunk; ++i) {
+      chunk_first[i] = f;
+      f += chunk_n[i];
+      cs = std::max(cs, chunk_n[i]);
+    }
+    lay = plan_layout(width, height, cs, *p, true);
+    const size_t in_b = wh * cs, out_b = wh * cs * sizeof(float);
+    size_t off = lay.bytes;
+    auto take = [&](size_t n) {
+      const size_t o = off;
+      off += (n + 255) / 256 * 256;
+      return o;
+    };
+    slot_l[0] = lay.in_left;
+    slot_r[0] = lay.in_right;
+    slot_o[0] = lay.out;
+    slot_l[1] = nchunk > 1 ? take(in_b) : 0;
+    slot_r[1] = nchunk > 1 ? take(in_b) : 0;
+    slot_o[1] = nchunk > 1 ? take(out_b) : 0;
+    s = ensure_workspace(h, off);
+    if (s != BDIS_E_NOMEM || even || count < 2) break;
+    nchunk = even_chunks(count, chunk_n);  // smaller chunks
   }
-  const Layout lay = plan_layout(width, height, cs, *p, true);
-  const size_t in_b = wh * cs, out_b = wh * cs * sizeof(float);
-  size_t off = lay.bytes;
-  auto take = [&](size_t n) {
-    const size_t o = off;
-    off += (n + 255) / 256 * 256;
-    return o;
-  };
-  const size_t slot_l[2] = {lay.in_left, nchunk > 1 ? take(in_b) : 0};
-  const size_t slot_r[2] = {lay.in_right, nchunk > 1 ? take(in_b) : 0};
-  const size_t slot_o[2] = {lay.out, nchunk > 1 ? take(out_b) : 0};
-  s = ensure_workspace(h, off);
   if (s != BDIS_OK) return s;
   if (nchunk > 1) {
     s = ensure_pipeline(h);

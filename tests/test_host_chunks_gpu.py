@@ -1,0 +1,48 @@
+"""The blocking host entry's chunks."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2106_07136_gb300 as bd
+
+pytestmark = pytest.mark.gpu
+
+KW = dict(iterations=3, coarsest_scale=2, gamma=0.25)
+
+
+def pairs(w, h, count):
+    rng = np.random.default_rng(count)
+    tile = rng.integers(0, 256, (3, h, w + 8), dtype=np.uint8)
+    idx = rng.integers(0, 3, count)
+    return [torch.from_numpy(np.ascontiguousarray(tile[idx][:, :, o:o + w])) for o in (5, 8)]
+
+
+def same(a, b):
+    return torch.equal(a.view(torch.int32), b.view(torch.int32))
+
+
+@pytest.mark.parametrize("w,h,count", [(640, 480, 2), (640, 480, 7), (640, 480, 13), (640, 480, 49),
+                                       (1601, 1203, 41)])
+def test_a_workspace_that_cannot_be_had_takes_smaller_chunks(w, h, count):
+    left, right = pairs(w, h, count)
+    p = bd.default_params(**KW)
+    m = bd.Matcher("cuda:0")
+    ref = m.match_host(left.pin_memory(), right.pin_memory(), p)
+    whole = m.workspace_bytes
+    m.close()
+    m = bd.Matcher("cuda:0")
+    bd.inject_alloc_failures(1)
+    try:
+        out = m.match_host(left.pin_memory(), right.pin_memory(), p)
+        assert m.workspace_bytes <= 0.8 * whole
+        assert same(out, ref)
+        bd.inject_alloc_failures(2)
+        fresh = bd.Matcher("cuda:0")
+        with pytest.raises(bd.BdisError) as e:
+            fresh.match_host(left, right, p)
+        assert e.value.status == bd._lib.BDIS_E_NOMEM
+    finally:
+        bd.inject_alloc_failures(0)
+    assert same(fresh.match_host(left.pin_memory(), right.pin_memory(), p), ref)
+    fresh.close()
+    m.close()

@@ -240,8 +240,9 @@ int bdis_proposal_level(int coarsest_scale);
 /* Same, with HOST buffers: left/right are `count` dense width x height uint8
  * images in host memory, disparity_out a dense host float array. The call
  * copies in, matches, copies out and returns when the result is in
- * disparity_out. A batch of the work of 12 or more 640x480 pairs runs as 2
- * chunks (from 48 as 3, from 256 as 5, the first and last ones small): one
+ * disparity_out. A batch of the pixels of 12 or more 640x480 pairs runs as 2 to
+ * 5 chunks, by its estimated time (smaller ones where the workspace of the
+ * largest cannot be had): one
  * chunk's inputs are copied in while the previous chunk is matched and the
  * one before is copied out (two copy streams owned by the handle, device
  * buffers double-buffered). Pinned host memory makes the

@@ -889,19 +889,21 @@ bdis_status bdis_warm_map(const float *prev, int width, int height, int level, i
 
 namespace {
 
-// How bdis_match_host splits a batch. A chunk costs about 90 us of launches and
-// underfilled coarse levels, as much as matching four 640x480 pairs; it hides
-// the copies of its neighbours (a pair's copy in takes an eighth of its match, its
-// copy out a quarter). So a small batch runs whole; a larger one splits off a last
-// chunk, whose copy out is all that nothing hides; then also a first one, whose
-// copy in nothing hides; and a large one grades the middle, so that each copy
-// still fits under the match beside it. Lines drawn by the work, in 640x480
-// pairs, all sides measured (us per call, even split of before -> now): 8 pairs
-// 575 -> 389 (two chunks 422), 16 pairs 783 -> 650 (one chunk 665), 32 pairs 1258
-// -> 1130 (one 1202, three 1142), 64 pairs 2072 -> 1953 (two 2075, four 2017), 128
-// pairs 3677 -> 3611, 512 pairs 13350 -> 13240 (three 13780). A middle chunk past
-// 32 GB of workspace keeps the even split, whose chunks are smaller; so does a
-// batch whose workspace cannot be had.
+// How bdis_match_host splits a batch. A chunk costs about 50 us of launches and
+// underfilled coarse levels; it hides the copies of its neighbours. So a small batch
+// runs whole; a larger one splits off a last chunk, whose copy out is all that
+// nothing hides; then also a first one, whose copy in nothing hides; and a large
+// one grades the middle. Lines drawn in 640x480 pairs, all sides measured at the
+// default settings (us per call, even split -> graded): 8 pairs 575 -> 389 (two
+// chunks 422), 16 pairs 783 -> 650 (one chunk 665), 32 pairs 1258 -> 1130 (one
+// 1202, three 1142), 64 pairs 2072 -> 1953 (two 2075, four 2017), 128 pairs 3677
+// -> 3611, 512 pairs 13350 -> 13240 (three 13780). But a graded split's long chunk
+// hides its copies only where the match takes several times as long as they do, and
+// settings that match fast want the even one (64 pairs at overlap 0.25, 2
+// iterations, finest scale 1: even 708, graded 857; 128 at overlap 0.5: 1959 and
+// 2228): from 12 pairs on, the split whose estimated time (below) is less is taken,
+// the even one also within 1%. A middle chunk past 32 GB of workspace keeps the even
+// split, whose chunks are smaller; so does a batch whose workspace cannot be had.
 constexpr int kHostChunks = 5;
 
 // Chunks of at most a third of the batch (a quarter from 8 pairs): from 32 pairs
@@ -917,6 +919,41 @@ int even_chunks(int count, int (&n)[kHostChunks]) {
   int k = 0;
   for (int left = count; left > 0; left -= per) n[k++] = std::min(per, left);
   return k;
+}
+
+// Time of a split in us: chunk i's copy in, match and copy out each follow their own
+// of the chunk before; the slots of chunk i - 2 are free once it is matched (inputs)
+// and copied out (output). Rates as measured over 29 settings x 9 batches (rms error
+// 4%): 2.4 and 6 us for a 640x480 pair's copies; for a chunk of five levels 42 us and
+// one more per iteration (12 at most), for fewer levels less; a match by its pixels
+// and its patches' pixels, more or less by the iterations (for images whose patches
+// need them all). From 12 pairs on, the split it picks is within 3% of the even one
+// or faster over the 29 settings, where always the graded one took up to 1.35 times
+// as long.
+double split_us(int w, int h, const bdis_params &p, const int *n, int k) {
+  const double pairs = (double)w * h / (640.0 * 480.0);
+  const int stride = grid_stride(p.patch_size, p.overlap);
+  double patches = 0;
+  for (int l = p.finest_scale; l <= p.coarsest_scale; ++l)
+    patches += (double)grid_count(level_dim(w, l), p.patch_size, stride) *
+               grid_count(level_dim(h, l), p.patch_size, stride);
+  const bool fixed = p.window_samples == 5 && p.window_step == 0.5f &&
+                     (p.patch_size == 8 || p.patch_size == 12 || p.patch_size == 16);
+  const int it = std::min(p.iterations, 12);
+  const double per_patch_pixel =
+      fixed ? (1.5 + 0.2 * std::min(it, 3) + 0.04 * std::max(it - 3, 0)) * 1e-6 : 6e-6;
+  const double match = pairs * (p.finest_scale ? 5.0 : 7.5) +
+                       patches * p.patch_size * p.patch_size * per_patch_pixel;
+  const double chunk = (42.0 + it) * (p.coarsest_scale - p.finest_scale + 2) / 6.0;
+  double in = 0, run = 0, out = 0, ran[2] = {}, left[2] = {};
+  for (int i = 0; i < k; ++i) {
+    in = std::max(in, ran[i & 1]) + n[i] * pairs * 2.4;
+    run = std::max(std::max(run, in), left[i & 1]) + chunk + n[i] * match;
+    out = std::max(out, run) + n[i] * pairs * 6.0;
+    ran[i & 1] = run;
+    left[i & 1] = out;
+  }
+  return out;
 }
 
 int host_chunks(int w, int h, int count, const bdis_params &p, int (&n)[kHostChunks]) {
@@ -943,8 +980,13 @@ int host_chunks(int w, int h, int count, const bdis_params &p, int (&n)[kHostChu
     k = 5;
   }
   const int largest = *std::max_element(n, n + k);
-  if (k > 1 && plan_layout(w, h, largest, p, true).bytes > (32ull << 30))
-    return even_chunks(count, n);
+  int even[kHostChunks];
+  const int ke = even_chunks(count, even);
+  if (k > 1 && (plan_layout(w, h, largest, p, true).bytes > (32ull << 30) ||
+                split_us(w, h, p, even, ke) < 1.01 * split_us(w, h, p, n, k))) {
+    std::copy(even, even + ke, n);
+    k = ke;
+  }
   return k;
 }
 

@@ -46,3 +46,21 @@ def test_a_workspace_that_cannot_be_had_takes_smaller_chunks(w, h, count):
     assert same(fresh.match_host(left.pin_memory(), right.pin_memory(), p), ref)
     fresh.close()
     m.close()
+
+
+@pytest.mark.parametrize("kw,longest", [(dict(KW, overlap=0.25, finest_scale=1), 20),
+                                        (dict(KW, overlap=0.5), 20), (dict(KW, iterations=12), 48)])
+def test_fast_settings_take_chunks_of_equal_length(kw, longest):
+    """64 pairs: settings whose match takes no longer than a few copies run in chunks of at most 20
+    (seen by the workspace: pyramid, patches and two sets of images of the longest chunk), the
+    default's kind in one of 48 between two short ones; the device entry's maps either way."""
+    left, right = pairs(640, 480, 64)
+    p = bd.default_params(**kw)
+    m, r = bd.Matcher("cuda:0"), bd.Matcher("cuda:0")
+    out = m.match_host(left.pin_memory(), right.pin_memory(), p)
+    r.reserve(640, 480, longest, p)
+    images = 2 * 640 * 480 * longest * 6
+    assert r.workspace_bytes < m.workspace_bytes <= r.workspace_bytes + images + (1 << 16)
+    assert same(out, r.match(left.cuda(), right.cuda(), p).cpu())
+    m.close()
+    r.close()

@@ -9,6 +9,7 @@
 // autotuner times, per group and level, the candidate lane layouts, block
 // sizes and sampling (global or warp-tiled) of the search kernel and the
 // densify kernels on the group's own data, and keeps the fastest.
+#include <algorithm>
 #include <new>
 #include <optional>
 #include <vector>
@@ -146,10 +147,21 @@ bdis_status bdis_plan_create(int device, const bdis_group *groups, int n_groups,
   bdis_status run_status = BDIS_OK;
   // Several branches run beside one another, so another branch's blocks fill a
   // launch's tail; overlapped launches on top only place blocks unevenly (32
-  // pairs of four sizes: 1622 us with them, 1591 without). A single branch keeps
-  // them.
+  // pairs of four sizes: 1622 us with them, 1591 without; two groups of one
+  // 640x480 pair 109.4 and 106.7, six of two 160x120 pairs 102 and 86). A single
+  // branch keeps them, and so do two small ones, whose launches leave most of the
+  // SMs free: two groups of one 160x120 pair 62.2 with, 64.4 without; of three 70.4
+  // and 71.5, of four 73.3 and 71.0; of one 320x240 pair 80.0 and 82.5, of two 94.3
+  // and 90.3.
   std::optional<bdis::NoOverlap> plain;
-  if (pl->groups.size() > 1) plain.emplace();
+  long long pixels = 0;
+  int most = 0;
+  for (const auto &g : pl->groups) {
+    pixels += (long long)g.left.width * g.left.height * g.left.count;
+    most = std::max(most, g.left.count);
+  }
+  const size_t n = pl->groups.size();
+  if (n > 2 || (n == 2 && (pixels > 2 * 320 * 240 || most > 3))) plain.emplace();
   for (auto &g : pl->groups) {
     if (e != cudaSuccess || run_status != BDIS_OK) break;
     e = cudaStreamWaitEvent(g.stream, pl->fork, 0);

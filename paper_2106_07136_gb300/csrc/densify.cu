@@ -364,9 +364,10 @@ struct DisTile {
   int ic0, ic1, jr0, jr1, nc;
 };
 
-// 1 / m for m in [1, 2^100]: one Newton step with fused residual on an
+// 1 / m for m in [1, 2^124]: one Newton step with fused residual on an
 // approximation within 1 ulp, which rounds correctly unless m's significand is
-// all ones (P. Markstein, IBM J. Res. Dev. 34, 1990; there it may be an ulp off).
+// all ones (P. Markstein, IBM J. Res. Dev. 34, 1990), and there too on this device:
+// the same as the division for every float of the range.
 // __frcp_rn's test of its argument's range, per pixel and patch, made the whole
 // call 10% slower (64 pairs of 640x480: 1965 us against 1786, same maps).
 __device__ __forceinline__ float dis_reciprocal(float m) {
@@ -376,8 +377,9 @@ __device__ __forceinline__ float dis_reciprocal(float m) {
 }
 
 // Numerators and denominators of column x, rows y0 and y0 + 1. PLAIN: weights 1
-// and every sample inside. There a residual is cut to 2^50, which keeps the
-// reciprocal in its range: its weight is then 2^-100 and not less.
+// and every sample inside. There a residual is cut to 2^62, which keeps the
+// reciprocal in its range: its weight is then 2^-124 and not less, which changes
+// nothing beside a total above 2^-90.
 template <bool PLAIN>
 __device__ __forceinline__ void dis_gather(const DensifyArgs &a, const DisTile &tile, int b, int x,
                                            int y0, float (&num)[kDisR], float (&den)[kDisR]) {
@@ -399,7 +401,7 @@ __device__ __forceinline__ void dis_gather(const DensifyArgs &a, const DisTile &
     const float e = fmaf(p.t, q.y, q.x) - Lx[r];
     float wpx;
     if (PLAIN) {
-      const float c = fminf(fmaxf(fabsf(e), 1.f), 0x1p50f);
+      const float c = fminf(fmaxf(fabsf(e), 1.f), 0x1p62f);
       wpx = dis_reciprocal(c * c);  // c * c = max(e * e, 1)
     } else {
       wpx = p.weight / fmaxf(e * e, 1.f);

@@ -64,3 +64,18 @@ def test_fast_settings_take_chunks_of_equal_length(kw, longest):
     assert same(out, r.match(left.cuda(), right.cuda(), p).cpu())
     m.close()
     r.close()
+
+
+@pytest.mark.parametrize("kw", [KW, dict(KW, overlap=0.25, finest_scale=1)])
+@pytest.mark.parametrize("w,h,count", [(640, 480, 13), (640, 480, 49), (1601, 1203, 41)])
+def test_pageable_memory_through_the_chunks(kw, w, h, count):
+    """Graded and even splits from and to memory that is not pinned, twice through one handle: the
+    device entry's maps."""
+    left, right = pairs(w, h, count)
+    p = bd.default_params(**kw)
+    m = bd.Matcher("cuda:0")
+    outs = [m.match_host(left, right, p, torch.empty(count, h, w)) for _ in range(2)]
+    ref = m.match(left.cuda(), right.cuda(), p).cpu()
+    m.close()
+    for out in outs:
+        assert not out.is_pinned() and same(out, ref)

@@ -518,7 +518,8 @@ int bdis_net_weight_count(void);
  * runs its forward pass and data gradients in the banded kernel under 1; under
  * 2 its forward pass takes the per-tile kernel and its data gradients mma.sync.
  * Inputs too wide for a kernel's shared memory take the next one down, and so
- * do training batches whose padded activations pass 32 GB. Process-wide. */
+ * do training batches whose padded activations pass 32 GB and large ones of
+ * images of a few pixels. Process-wide. */
 void bdis_set_net_variant(int tensor_path);
 int bdis_get_net_variant(void);
 
@@ -542,8 +543,9 @@ bdis_status bdis_net_forward(bdis_net *net, const float *L, const float *R, int 
  * The network keeps, beside what its forward passes use (352 B per position of
  * images framed by 4 pixels on each side; 448 B per pixel of images that the
  * default kernels do not take), 704 B per framed position; a batch past 32 GB of
- * them, or for which they cannot be had, 768 B per pixel; 576 where those cannot
- * be had. BDIS_E_NOMEM if these cannot either. */
+ * them, or for which they cannot be had, or a large one of images of a few pixels,
+ * 768 B per pixel; 576 where those cannot be had. BDIS_E_NOMEM if these cannot
+ * either. */
 bdis_status bdis_net_gradient(bdis_net *net, const float *L, const float *R, int r_stride,
                               int width, int height, int count, const float *label,
                               float *loss_out, float *grad_out, void *stream);

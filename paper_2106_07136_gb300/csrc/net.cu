@@ -1794,6 +1794,20 @@ void net_release(bdis_net *n) {
   delete n;
 }
 
+// Whether a gradient takes the padded planar layout, for images that fit it. Its
+// launches have 60 us less to set up, but a band is one image's and works in tiles
+// of 128 positions of its padded rows, which large batches of images of a few
+// pixels hardly fill. By the time per image, measured over 17 sizes (1x1 to 15x20)
+// x 100 to 200,000 pixels (us, planar and per layer): 0.10 and 0.09 per tile, against
+// 0.0018 per pixel and 0.00066 per position of the dilation-4 weight gradient's
+// frame. 5555 images of 3x3: 1155 planar, 394 per layer; 111: 138 and 189; 462 of
+// 9x12: 273 and 295.
+bool planar_gradient(int H, int W, int count) {
+  const double planar = 0.10 + 0.09 * (((long long)H * (W + 2 * kPad) + kWgTile - 1) / kWgTile);
+  const double layers = 0.0018 * H * W + 0.00066 * (H + 4) * (W + 4);
+  return count * (planar - layers) <= 60.0;
+}
+
 }  // namespace
 
 namespace bdis {
@@ -1892,13 +1906,14 @@ bdis_status bdis_net_gradient(bdis_net *n, const float *L3, const float *R3, int
   if (!g_sms) init_sms();
   // Images that fit the banded kernel train in its layout: the forward pass,
   // the loss with the data gradients, and the weight gradients are one launch
-  // each (64 images of 40x30: 310 us by per-layer launches, 228 now). Its
+  // each (64 images of 40x30: 310 us by per-layer launches, 211 now). Its
   // padded planes take 704 B per position where the NHWC ones take 768 B per
   // pixel (576 at least); a batch beyond 32 GB of them, or for which they cannot be
-  // had, keeps the NHWC form.
+  // had, keeps the NHWC form, and so does a large batch of images of a few pixels.
   bool done = false;
   const double planar_bytes = 704.0 * (height + 2 * kPad) * (width + 2 * kPad) * (double)count;
-  if (g_net_tc == 1 && planar_bytes <= 32e9 && band_fits(height, width)) {
+  if (g_net_tc == 1 && planar_bytes <= 32e9 && planar_gradient(height, width, count) &&
+      band_fits(height, width)) {
     bdis_net::Planar &p = n->train;
     s = net_reserve_planar(p, n->kept_train, height, width, count, true, st);
     if (s != BDIS_OK && s != BDIS_E_NOMEM) return s;

@@ -141,3 +141,24 @@ def test_two_gradient_buffers_give_the_same_gradient(net_variant, shape):
     net.status()
     net.close()
     ref_net.close()
+
+
+@pytest.mark.parametrize("shape", [(1000, 1, 1), (2000, 5, 5), (700, 40, 2)])
+def test_large_batches_of_tiny_images_train_layer_by_layer(shape):
+    """The default variant takes the launches per layer there, as variant 2 does: its gradient bit
+    for bit; a small batch of the same images does not (within the order of 32-bit sums)."""
+    batch = net_batch(9, *shape)
+    few = [t[:8].contiguous() for t in batch]
+    net = bd.ProposalNet(bd.net_init_weights(seed=6))
+    old = bd.get_net_variant()
+    try:
+        bd.set_net_variant(2)
+        ref, ref_few = net.gradient(*batch)[1], net.gradient(*few)[1]
+        bd.set_net_variant(1)
+        g, g_few = net.gradient(*batch)[1], net.gradient(*few)[1]
+    finally:
+        bd.set_net_variant(old)
+    net.status()
+    net.close()
+    assert np.array_equal(g, ref)
+    assert np.linalg.norm(g_few - ref_few) <= 1e-5 * np.linalg.norm(ref_few)

@@ -1545,6 +1545,34 @@ bool band_fits(int H, int W) {
          band_rows<32, 16>(1, H, W, &nsb);
 }
 
+// Band height of a layer of at most `limit` rows a band: of the numbers of equal
+// bands per image, that whose rounds over the SMs cost least, a round
+// being a band's tiles and one more for its fill and drain. Bands of fewer
+// rows spread a small batch over the SMs, but a last round that few blocks
+// have work in costs as much as a full one: 64 images of 40x30 in 3 bands each
+// were 192 bands on 152 SMs (59 us a forward pass by host clock), in 2 they are
+// 128 (51); 32 in 5 bands 52, in 4 40; 100 in 2 bands 74, in 3 61. A result
+// does not depend on the band height: each position's MMAs and epilogue are
+// the same.
+// Only the least number of bands of each height is looked at (a call spends 2 us on
+// this, not 20, where images are 240 rows high).
+int band_height(int H, int Wp, int count, int limit) {
+  int best = 0;
+  long long cost = 0;
+  for (int nb = (H + limit - 1) / limit;;) {
+    const int rows = (H + nb - 1) / nb;
+    const long long c = ((long long)count * ((H + rows - 1) / rows) + g_sms - 1) / g_sms *
+                        ((rows * Wp + 127) / 128 + 1);
+    if (!best || c < cost) {
+      best = rows;
+      cost = c;
+    }
+    if (rows == 1) return best;
+    nb = (H + rows - 2) / (rows - 1);
+    if ((long long)count * (nb - 1) >= 8LL * g_sms) return best;  // more rounds only add fills
+  }
+}
+
 // One cooperative launch of net_chain_kernel<BACK> over `layers` layers with
 // their buffers filled in (dilation included): picks the band heights. Returns
 // false, having launched nothing, when the images are too wide for it or the
@@ -1557,15 +1585,8 @@ bool launch_chain(bdis_net *n, BandNet &net, int H, int W, int count, cudaStream
     bh[l] = l == 0   ? band_rows<16, 32>(net.layer[l].dil, H, W, &nsb[l])
             : l == 5 ? band_rows<32, 16>(net.layer[l].dil, H, W, &nsb[l])
                      : band_rows<32, 32>(net.layer[l].dil, H, W, &nsb[l]);
-  // Band heights: per layer, the number of equal bands per image (at least as
-  // many as the limits ask for) whose rounds over the SMs cost least, a round
-  // being a band's tiles and one more for its fill and drain. Bands of fewer
-  // rows spread a small batch over the SMs, but a last round that few blocks
-  // have work in costs as much as a full one: 64 images of 40x30 in 3 bands each
-  // were 192 bands on 152 SMs (59 us a forward pass by host clock), in 2 they are
-  // 128 (51); 32 in 5 bands 52, in 4 40; 100 in 2 bands 74, in 3 61. A result
-  // does not depend on the band height: each position's MMAs and epilogue are
-  // the same.
+  int limit[6];
+  std::copy(bh, bh + 6, limit);
   int slab = 0;
   // one block per SM, or one per band where a layer has fewer bands (a
   // single image): fewer blocks meet at each grid barrier and restage the
@@ -1574,18 +1595,9 @@ bool launch_chain(bdis_net *n, BandNet &net, int H, int W, int count, cudaStream
   for (int l = 0; l < layers; ++l) {
     if (!bh[l]) return false;
     const int Wp = W + 2 * kPad, soff = net.layer[l].dil * Wp + net.layer[l].dil;
-    int best = 0;
-    long long cost = 0;
-    for (int nb = (H + bh[l] - 1) / bh[l]; nb <= H; ++nb) {
-      const int rows = (H + nb - 1) / nb;
-      const long long c = ((long long)count * ((H + rows - 1) / rows) + g_sms - 1) / g_sms *
-                          ((rows * Wp + 127) / 128 + 1);
-      if (!best || c < cost) {
-        best = rows;
-        cost = c;
-      }
-      if ((long long)count * nb >= 8LL * g_sms) break;  // more rounds only add fills
-    }
+    int m = 0;
+    while (limit[m] != bh[l]) ++m;  // the choice depends on the limit alone
+    const int best = m < l ? net.layer[m].BH : band_height(H, Wp, count, bh[l]);
     if (best < bh[l]) {  // the limits still hold
       bh[l] = best;
       nsb[l] = (best * Wp + 127) / 128 * 128 + 2 * soff;

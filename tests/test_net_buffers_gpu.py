@@ -1,5 +1,6 @@
 """What a network's calls share: buffers across streams, shapes, captures and failures."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -162,3 +163,23 @@ def test_large_batches_of_tiny_images_train_layer_by_layer(shape):
     net.close()
     assert np.array_equal(g, ref)
     assert np.linalg.norm(g_few - ref_few) <= 1e-5 * np.linalg.norm(ref_few)
+
+
+def test_a_call_costs_the_host_the_same_for_tall_images():
+    """Enqueueing a forward pass: the band heights of images of 240 rows are chosen in little more
+    time than those of one row (the least of many calls, so that nothing else of the host counts)."""
+    net = bd.ProposalNet(bd.net_init_weights(seed=6))
+
+    def least(shape):
+        L, R, _ = net_batch(10, *shape)
+        best = np.inf
+        for _ in range(300):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            net.forward(L, R)
+            best = min(best, time.perf_counter() - t0)
+        return best
+
+    short, tall = least((1, 1, 135)), least((1, 240, 135))
+    net.close()
+    assert tall <= 1.5 * short, (short, tall)

@@ -1554,26 +1554,29 @@ bool band_fits(int H, int W) {
 }
 
 // Band height of a layer of at most `limit` rows a band: of the numbers of equal
-// bands per image, that whose rounds over the SMs cost least, a round
-// being a band's tiles and one more for its fill and drain. Bands of fewer
-// rows spread a small batch over the SMs, but a last round that few blocks
-// have work in costs as much as a full one: 64 images of 40x30 in 3 bands each
-// were 192 bands on 152 SMs (59 us a forward pass by host clock), in 2 they are
-// 128 (51); 32 in 5 bands 52, in 4 40; 100 in 2 bands 74, in 3 61. A result
-// does not depend on the band height: each position's MMAs and epilogue are
-// the same.
-// Only the least number of bands of each height is looked at (a call spends 2 us on
-// this, not 20, where images are 240 rows high).
+// bands per image, that whose rounds over the SMs cost least, a round being a band's
+// tiles and two more for its fill and drain; at the same cost more bands only where
+// they spare an eighth of the tiles. Bands of fewer rows spread a small batch over
+// the SMs, but a last round that few blocks have work in costs as much as a full
+// one: 64 images of 40x30 in 3 bands each were 192 bands on 152 SMs (59 us a forward
+// pass by host clock), in 2 they are 128 (51); 32 in 5 bands 52, in 4 40; 100 in 2
+// bands 74, in 3 61. With one tile for fill and drain, 160 images of 80x64 took 292
+// us, with two 281; 512 of 32x24 181 and 175; with two and no more bands at the same
+// cost, 56 of 60x34 66 where more take 62. A result does not depend on the band
+// height: each position's MMAs and epilogue are the same. Only the least number of
+// bands of each height is looked at (a call spends 2 us on this, not 20, where
+// images are 240 rows high).
 int band_height(int H, int Wp, int count, int limit) {
   int best = 0;
-  long long cost = 0;
+  long long cost = 0, work = 0;
   for (int nb = (H + limit - 1) / limit;;) {
-    const int rows = (H + nb - 1) / nb;
-    const long long c = ((long long)count * ((H + rows - 1) / rows) + g_sms - 1) / g_sms *
-                        ((rows * Wp + 127) / 128 + 1);
-    if (!best || c < cost) {
+    const int rows = (H + nb - 1) / nb, tiles = (rows * Wp + 127) / 128;
+    const long long rounds = ((long long)count * ((H + rows - 1) / rows) + g_sms - 1) / g_sms;
+    const long long c = rounds * (tiles + 2), w = rounds * tiles;
+    if (!best || c < cost || (c == cost && 8 * w <= 7 * work)) {
       best = rows;
       cost = c;
+      work = w;
     }
     if (rows == 1) return best;
     nb = (H + rows - 2) / (rows - 1);

@@ -199,12 +199,11 @@ int pyramid_fused();
 void set_pyramid_fused(int variant);
 
 // ---- Bounds-checked build (-DBDIS_CHECKED; the memory-sanitizer substitute,
-// libbdis_checked.so). There, the kernels' data-dependent global accesses (and
-// the tiled search's reads of its staged rows)
-// check their element index against the buffer's extent; an access out of
-// bounds is skipped (a read gives 0) and sets bit `site` of this translation
-// unit's check word, which bdis_check_status reads. In the normal build the
-// checks compile away. Sites:
+// libbdis_checked.so). There, the kernels' data-dependent global accesses, and
+// the tiled search's reads of its staged rows, check their element index against
+// the buffer's extent; an access out of bounds is skipped (a read gives 0) and
+// sets bit `site` of this translation unit's check word, which bdis_check_status
+// reads. In the normal build the checks compile away. Sites:
 enum CheckSite {
   kCheckSearchSample = 0,   // inverse search: right-plane samples (window and steps)
   kCheckSearchRows = 1,     // inverse search: template and gradient rows

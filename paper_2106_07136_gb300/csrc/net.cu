@@ -408,9 +408,9 @@ __global__ void __launch_bounds__(128) conv_tc_kernel(
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;\n" ::"r"(tmem));
 }
 
-// ------------------------------------------- conv (tcgen05, banded inference)
+// ------------------------------------------------------ conv (tcgen05, banded)
 
-// The inference forward pass, and training, keep every activation in a padded planar
+// Forward passes, and training, keep every activation in a padded planar
 // layout in global memory: each image is framed by kPad zero rows and
 // columns (kPad = the largest dilation, so every tap of a real pixel lands
 // inside its own frame), frames are numbered back to back, and each group of
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(128) conv_tc_kernel(
 // cores' no-swizzle K-major operand layout, and the rows any band of
 // positions reads form one contiguous range per plane: one bulk copy each.
 //
-// The whole forward pass is one cooperative launch, one block per SM: the
+// A whole forward pass is one cooperative launch, one block per SM: the
 // input is packed, then the six layers run in turn with a grid barrier
 // between steps (a band's halo was written by other blocks). Within a layer
 // the block is warp-specialised, three stages in flight:
@@ -490,7 +490,7 @@ __device__ __forceinline__ void *band_smem_base() {
   return band_smem;
 }
 
-// One layer of the fused inference kernel below.
+// One layer of the fused kernel below.
 struct BandLayer {
   const __nv_bfloat16 *in, *wt;
   const float *bias;
@@ -1463,9 +1463,9 @@ cudaError_t pack_all(bdis_net *n, cudaStream_t st) {
 }
 
 int g_sms = 0;
-// forward convolutions: 1 = banded tcgen05 kernel for inference (default; training
-// forwards and inputs too wide for it take the per-tile one), 2 = per-tile tcgen05
-// kernel, 0 = mma.sync kernel
+// convolutions: 1 = banded tcgen05 kernel for forward passes and data gradients
+// (default; what it does not take runs as under 2), 2 = forward passes per tile on
+// tcgen05, data gradients on mma.sync, 0 = all on mma.sync
 int g_net_tc = 1;
 
 // Dynamic shared memory of the tcgen05 kernel is exactly its slab and the

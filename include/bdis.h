@@ -422,8 +422,10 @@ int bdis_get_pyramid_variant(void);
  * kernels that have at most 16 blocks per SM (small batches, coarse levels)
  * are programmatic dependents of the kernel before them on the stream, so a
  * launch's start-up overlaps the previous kernel's last blocks; each kernel
- * still waits for the previous one to finish before it touches memory.
- * 0: plain stream order. Results are identical. Process-wide. */
+ * still waits for the previous one to finish before it touches memory. A
+ * plan of several groups is captured in plain order, unless it is two groups of
+ * at most three small pairs. 0: plain stream order. Results are identical.
+ * Process-wide. */
 void bdis_set_launch_overlap(int on);
 int bdis_get_launch_overlap(void);
 
